@@ -188,6 +188,12 @@ size_t rsi_stage_workspace_bytes(const rsi_stage *st, int64_t n_src, int64_t n_t
  *   PISTON  field[j] = -(v0 / 2 pi) sum_i w_i e^{ikr_ij} / r_ij
  *   RSI     field[j] = -(i / lambda) sum_i w_i sigma_i e^{ikr}/r (1 - 1/(ikr)) cos(theta_ij)
  * with lambda = 2 pi / k.  Pairs closer than 1e-12 m contribute nothing.
+ * FP32C with nothing asked for (tile, tpt and variant 0) and a long sum: the
+ * device may take clusters of sources and of targets that are far apart
+ * together, through Chebyshev nodes of their rectangles, where its estimate of
+ * the work says that this is faster; a pair of clusters is then interpolated to
+ * 5e-7 of a term at most (5e-8 root mean square), below the FP32 rounding of a
+ * pair.  variant 3 asks for the direct sum.
  * src_sigma: complex [n_src] in the source set's slot order (RSI only; NULL
  * for PISTON).  tgt_field: complex [n_tgt] in the target set's slot order,
  * overwritten.  workspace: >= rsi_stage_workspace_bytes(...), 256-byte
@@ -214,7 +220,8 @@ int rsi_propagate_stage(const rsi_stage *st,
  * another (k_j = 2 k_i to a relative 2^-40; with one sound speed, one
  * frequency twice another), e^{i k_j (r - R)} is formed from e^{i k_i (r - R)}
  * by the double angle on pairs away from the tile, two MUFU operations per
- * pair fewer.  The doubled angle carries twice the sincos's angle error: on
+ * pair fewer (in the direct sum; clusters, as in rsi_propagate_stage, are taken
+ * frequency by frequency).  The doubled angle carries twice the sincos's angle error: on
  * 2.25, 5 and 10 MHz the 10 MHz image is 9.7e-7 from the FP64 oracle (5.5e-7
  * with its own sincos), far inside the FP32C tolerance.                    */
 size_t rsi_stage_multi_workspace_bytes(const rsi_stage *st, int32_t nf, const double *ks, int64_t n_src,
@@ -240,7 +247,8 @@ int rsi_stage_multi_shared_harmonic(const rsi_stage *st, int32_t nf, const doubl
  *     sources fit), 48 bytes with per-point normals (1.4 million) and 64
  *     bytes for FP64 (1.0 million) -- plus, when the sources are split
  *     across CTAs, 16 bytes per target for every split.  A stage that does
- *     not fit is rejected with RSI_E_NOMEM before anything is enqueued.  With
+ *     not fit is rejected with RSI_E_NOMEM before anything is enqueued.  The
+ *     direct sum is taken where the tables of the clusters would not fit.  With
  *     splits = 0 the call first lowers the automatic split count to what
  *     fits (chosen, below that bound, as rsi_propagate_stage chooses it).
  *   - The first call on a device looks up the area's device address (with
@@ -342,7 +350,8 @@ int rsi_field_image_sum(const rsi_grid *g, const double *field_a, const double *
 /* Times the FP32C launch shapes of one stage on the given data -- tile size
  * (32 ... 512, capped by the accuracy rule of at most n_src/64 sources per
  * tile) x targets per thread {2, 4} x distance update {reciprocal, Newton},
- * each shape needing at most workspace_bytes -- and writes the fastest to
+ * each shape needing at most workspace_bytes, and the automatic shape where
+ * that may take clusters -- and writes the fastest to
  * *best (kind, precision, k, v0 and normals copied from *st, splits = 0).
  * Each candidate runs once to warm up and twice timed (CUDA events on
  * `stream`); the call synchronises `stream` and leaves the last candidate's

@@ -113,7 +113,7 @@ __global__ void batch_grid_kernel(const BGrid* __restrict__ grids, const BSeg* _
 }
 
 __global__ void batch_prep_kernel(const BPrep* __restrict__ preps, const BPrepTile* __restrict__ tiles, int packed) {
-    __shared__ double red[32];
+    __shared__ __align__(8) float red[192];
     const BPrepTile t = tiles[blockIdx.x];
     const BPrep& p = preps[t.inst];
     // all instances share the CTA size; tiles of smaller instances use fewer

@@ -4,6 +4,7 @@
 // (step a6).
 #include <math.h>
 
+#include <algorithm>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -92,22 +93,10 @@ namespace {
 
 __global__ void reduce_partials_kernel(const double2* __restrict__ part, int splits, int64_t n,
                                        double2* __restrict__ out, int* status) {
-    int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (j >= n) return;
-    // Neumaier summation over the splits in index order
-    double sr = 0.0, cr = 0.0, si = 0.0, ci = 0.0;
-    for (int s = 0; s < splits; ++s) {
-        double2 v = part[size_t(s) * size_t(n) + size_t(j)];
-        double t = sr + v.x;
-        cr += (fabs(sr) >= fabs(v.x)) ? (sr - t) + v.x : (v.x - t) + sr;
-        sr = t;
-        t = si + v.y;
-        ci += (fabs(si) >= fabs(v.y)) ? (si - t) + v.y : (v.y - t) + si;
-        si = t;
-    }
-    double re = sr + cr, im = si + ci;
-    if (!isfinite(re) || !isfinite(im)) atomicExch(status, RSI_DEV_NONFINITE);
-    out[j] = make_double2(re, im);
+    reduce_partials(part, splits, n, out, status);
+}
+__global__ void reduce_gated_kernel(StageArgs a, double2* __restrict__ out) {
+    if (!gate_clustered(a.gate, a.S, a.gate_ratio)) reduce_partials(a.out, a.splits, a.n_tgt, out, a.status);
 }
 
 size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
@@ -115,6 +104,12 @@ size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
 struct Plan {
     int S, tpt, variant, splits, tiles_per_split, n_tiles;
     size_t tile_bytes, tiles_bytes, partial_bytes;
+    // the clustered kernel beside the direct one (the device chooses)
+    bool clustered;
+    ClusterPlan c;
+    // the direct kernel reads the clustered one's tiles; its partial sums follow everything else
+    size_t part_at() const { return clustered ? c.total() : tiles_bytes; }
+    size_t bytes() const { return part_at() + partial_bytes; }
 };
 
 bool valid_tile(int S) { return S == 32 || S == 64 || S == 128 || S == 256 || S == 512; }
@@ -178,14 +173,21 @@ int make_plan(const rsi_stage& st, int64_t n_src, int64_t n_tgt, Plan& p, int ma
         probe.tile_bytes = p.tile_bytes;
         int occ = fp32 ? stage_occupancy_fp32(probe) : stage_occupancy_fp64(probe);
         int64_t slots = int64_t(rsi_num_sms()) * occ;
-        // minimise (waves x tiles per CTA), the time of the busiest SM
-        int64_t best_cost = INT64_MAX;
+        // minimise (waves x tiles per CTA), the time of the busiest SM, plus
+        // the reduction: a CTA's tile takes S pairs per target at this GPU's
+        // pair rate (FP32C 1.4e12 / s over all slots), a split's partial sums 14
+        // FP64 operations per target at 2 a cycle and SM, on as many SMs as the
+        // reduction has CTAs.  2^16 x 2^14 (RSI, FP32C): 128 splits 744 + 137 us,
+        // 14 splits 827 + 19 us; a 1000 x 3000 x 1073 chain 218 -> 150 us
+        const double tile_us = double(p.S) * threads * p.tpt * double(slots) / (fp32 ? 1.4e6 : 7.5e3);
+        const double red_us = double(n_tgt) * 14.0 / (double(std::min<int64_t>(rsi_num_sms(), (n_tgt + 255) / 256)) * 4.1e3);
+        double best_cost = INFINITY;
         splits = 1;
         for (int s = 1; s <= max_auto_splits && s <= p.n_tiles; ++s) {
             int64_t tps = (p.n_tiles + s - 1) / s;
             int64_t s_act = (p.n_tiles + tps - 1) / tps;
             int64_t waves = (blocks * s_act + slots - 1) / slots;
-            int64_t cost = waves * tps;
+            const double cost = double(waves * tps) * tile_us + (s_act > 1 ? double(s_act) * red_us : 0.0);
             if (cost < best_cost) {
                 best_cost = cost;
                 splits = int(s_act);
@@ -197,6 +199,10 @@ int make_plan(const rsi_stage& st, int64_t n_src, int64_t n_tgt, Plan& p, int ma
     p.tiles_per_split = (p.n_tiles + splits - 1) / splits;
     p.splits = (p.n_tiles + p.tiles_per_split - 1) / p.tiles_per_split;
     p.partial_bytes = p.splits > 1 ? align256(size_t(p.splits) * size_t(n_tgt) * sizeof(double2)) : 0;
+
+    // the clustered kernel is offered where nothing about the launch shape is asked for
+    p.clustered = fp32 && !st.variant && !st.tile && !st.tpt &&
+                  cluster_plan(st.kind, st.normals, 1, n_src, n_tgt, p.S, st.splits, max_auto_splits, p.c);
     return RSI_OK;
 }
 
@@ -206,7 +212,7 @@ extern "C" size_t rsi_stage_workspace_bytes(const rsi_stage* st, int64_t n_src, 
     if (!st) return 0;
     Plan p;
     if (make_plan(*st, n_src, n_tgt, p) != RSI_OK) return 0;
-    return p.tiles_bytes + p.partial_bytes;
+    return p.bytes();
 }
 
 size_t rsi_stage_workspace_bytes_capped(const rsi_stage* st, int64_t n_src, int64_t n_tgt, int max_splits,
@@ -215,7 +221,7 @@ size_t rsi_stage_workspace_bytes_capped(const rsi_stage* st, int64_t n_src, int6
     Plan p;
     if (make_plan(*st, n_src, n_tgt, p, max_splits) != RSI_OK) return 0;
     if (splits) *splits = p.splits;
-    return p.tiles_bytes + p.partial_bytes;
+    return p.bytes();
 }
 
 extern "C" int rsi_propagate_stage(const rsi_stage* st, const void* src_points, int64_t n_src,
@@ -235,9 +241,8 @@ extern "C" int rsi_propagate_stage(const rsi_stage* st, const void* src_points, 
     Plan p;
     int rc = make_plan(*st, n_src, n_tgt, p);
     if (rc != RSI_OK) return rc;
-    if (workspace_bytes < p.tiles_bytes + p.partial_bytes)
-        return rsi_fail(RSI_E_NOMEM, "rsi_propagate_stage: workspace %zu < %zu bytes", workspace_bytes,
-                        p.tiles_bytes + p.partial_bytes);
+    if (workspace_bytes < p.bytes())
+        return rsi_fail(RSI_E_NOMEM, "rsi_propagate_stage: workspace %zu < %zu bytes", workspace_bytes, p.bytes());
     int* status = rsi_status_ptr();
     if (!status) return RSI_E_CUDA;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -246,10 +251,6 @@ extern "C" int rsi_propagate_stage(const rsi_stage* st, const void* src_points, 
     PointsView tgt = rsi_points_view(const_cast<void*>(tgt_points), n_tgt);
     uint8_t* tiles = static_cast<uint8_t*>(workspace);
     const double2* sigma = reinterpret_cast<const double2*>(src_sigma);
-    rc = fp32 ? launch_prep_fp32(*st, src, n_src, sigma, p.S, tiles, p.tile_bytes, p.n_tiles, s, p.variant == 3)
-              : launch_prep_fp64(*st, src, n_src, sigma, p.S, tiles, p.tile_bytes, p.n_tiles, s);
-    if (rc != RSI_OK) return rc;
-
     StageArgs a = {};
     a.kind = st->kind;
     a.normals = st->kind == RSI_STAGE_RSI ? base_normals(st->normals) : RSI_NORMALS_Z;
@@ -268,8 +269,24 @@ extern "C" int rsi_propagate_stage(const rsi_stage* st, const void* src_points, 
     a.kl = float(st->k - double(a.kh));
     a.tp = two_pi_split();
     double2* field = reinterpret_cast<double2*>(tgt_field);
-    a.out = p.splits > 1 ? reinterpret_cast<double2*>(tiles + p.tiles_bytes) : field;
+    a.out = p.splits > 1 ? reinterpret_cast<double2*>(tiles + p.part_at()) : field;
     a.status = status;
+    if (p.clustered) {
+        ClusterArgs c;
+        rc = cluster_prepare(*st, &st->k, 1.0f, src, n_src, sigma, a.tgt, n_tgt, field, p.c, tiles, status, c, s);
+        if (rc != RSI_OK) return rc;
+        a.gate = c.gate;
+        a.gate_ratio = c.gate_ratio;
+        TimingScope tsc = timing_begin(s);
+        rc = cluster_run(c, s);
+        if (rc == RSI_OK) rc = launch_stage_fp32(a, s);
+        if (rc != RSI_OK) return rc;
+        timing_end(tsc, st->kind, double(n_src) * double(n_tgt), s);
+        return p.splits > 1 ? launch_reduce_gated(a, field, s) : RSI_OK;
+    }
+    rc = fp32 ? launch_prep_fp32(*st, src, n_src, sigma, p.S, tiles, p.tile_bytes, p.n_tiles, s, p.variant == 3)
+              : launch_prep_fp64(*st, src, n_src, sigma, p.S, tiles, p.tile_bytes, p.n_tiles, s);
+    if (rc != RSI_OK) return rc;
     TimingScope tsc = timing_begin(s);
     rc = fp32 ? launch_stage_fp32(a, s) : launch_stage_fp64(a, s);
     if (rc != RSI_OK) return rc;
@@ -302,6 +319,12 @@ int launch_reduce_partials(const double2* part, int splits, int64_t n, double2* 
     unsigned blocks = unsigned((n + threads - 1) / threads);
     reduce_partials_kernel<<<blocks, threads, 0, s>>>(part, splits, n, out, status);
     RSI_CHECK_LAUNCH("reduce_partials_kernel");
+    return RSI_OK;
+}
+
+int launch_reduce_gated(const StageArgs& a, double2* out, cudaStream_t s) {
+    reduce_gated_kernel<<<unsigned((a.n_tgt + 255) / 256), 256, 0, s>>>(a, out);
+    RSI_CHECK_LAUNCH("reduce_gated_kernel");
     return RSI_OK;
 }
 
@@ -355,13 +378,15 @@ extern "C" int rsi_autotune_stage(const rsi_stage* st, const void* src_points, i
     RSI_CUDA_TRY(cudaEventCreate(&e1), "cudaEventCreate");
     float best_ms = 1e30f;
     rsi_stage win = base;
-    for (int S = 32; S <= cap; S <<= 1)
+    // S = 0: the automatic shape, where that may be the clustered kernel
+    for (int S = p0.clustered ? 0 : 32; S <= cap; S = S ? S << 1 : 32)
         for (int tpt : {1, 2, 4})
             for (int var : {1, 2, 3}) {
+                if (!S && (tpt > 1 || var > 1)) continue;
                 rsi_stage c = base;
                 c.tile = S;
-                c.tpt = tpt;
-                c.variant = var;
+                c.tpt = S ? tpt : 0;
+                c.variant = S ? var : 0;
                 if (rsi_stage_workspace_bytes(&c, n_src, n_tgt) > workspace_bytes) continue;
                 float t_best = 1e30f;
                 for (int rep = 0; rep < 3; ++rep) {

@@ -31,6 +31,46 @@ struct TwoPiSplit {
 };
 TwoPiSplit two_pi_split();
 
+// What the device decides for one stage (written by the clustered kernel's
+// preparation, stage_cluster_body.cuh)
+struct StageGate {
+    int L, h;                  // rows of the target set and strip height of the block order
+    unsigned long long cost;   // estimated instructions of the clustered kernel over the sampled pairs
+    unsigned long long pairs;  // samples: a tile and a quarter block (256 targets) each
+};
+// Which of the two kernels runs: the clustered kernel's estimated instructions
+// per warp, over all the stage's frequencies, against the direct sum's (16.8
+// per 32 pairs, 256 S pairs), which issues them 1.5 times as fast.  `ratio`: a
+// multi-frequency stage's instructions per frequency over a single stage's,
+// times the share of the GPU that the clustered kernel's CTAs fill.  On a
+// laminate's stages 0.5 mm apart, where the estimate is 0.6 of the direct sum's
+// instructions and 0.84 of the GPU is filled, both take 3.1 ms (2^16 x 2^16, 5
+// MHz).  FP32 arithmetic on integers: the same in every thread of both kernels.
+__device__ __forceinline__ bool gate_clustered(const StageGate* g, int S, float ratio) {
+    return float(g->cost) * 1.5f < float(g->pairs) * (134.4f * float(S)) * ratio;
+}
+
+// out[j] = sum over splits of part[split][j], j = this thread
+__device__ __forceinline__ void reduce_partials(const double2* __restrict__ part, int splits, int64_t n,
+                                                double2* __restrict__ out, int* status) {
+    int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (j >= n) return;
+    // Neumaier summation over the splits in index order
+    double sr = 0.0, cr = 0.0, si = 0.0, ci = 0.0;
+    for (int s = 0; s < splits; ++s) {
+        double2 v = part[size_t(s) * size_t(n) + size_t(j)];
+        double t = sr + v.x;
+        cr += (fabs(sr) >= fabs(v.x)) ? (sr - t) + v.x : (v.x - t) + sr;
+        sr = t;
+        t = si + v.y;
+        ci += (fabs(si) >= fabs(v.y)) ? (si - t) + v.y : (v.y - t) + si;
+        si = t;
+    }
+    double re = sr + cr, im = si + ci;
+    if (!isfinite(re) || !isfinite(im)) atomicExch(status, RSI_DEV_NONFINITE);
+    out[j] = make_double2(re, im);
+}
+
 struct StageArgs {
     int kind;      // RSI_STAGE_*
     int normals;   // RSI_NORMALS_*
@@ -49,6 +89,10 @@ struct StageArgs {
     TwoPiSplit tp;
     double2* out;  // [splits][n_tgt] partials, or the field when splits == 1
     int* status;
+    // where the clustered kernel is launched as well: the device's choice
+    // between them; null: this kernel runs
+    const StageGate* gate;
+    float gate_ratio;
 };
 
 size_t fp32_record_bytes(int kind, int normals);
@@ -67,6 +111,50 @@ int launch_prep_fp32(const rsi_stage& st, const PointsView& src, int64_t n_src, 
                      int S, uint8_t* tiles, size_t tile_bytes, int n_tiles, cudaStream_t s, bool packed = false);
 int launch_prep_fp64(const rsi_stage& st, const PointsView& src, int64_t n_src, const double2* sigma,
                      int S, uint8_t* tiles, size_t tile_bytes, int n_tiles, cudaStream_t s);
+// Clustered FP32C kernel (stage_cluster.cu), for up to 4 frequencies of a stage
+// at once.  Its workspace: per frequency the packed tiles, then `extra` (the
+// clusters and the rectangles of the targets, the gate last), then per
+// frequency the partial sums.
+constexpr int kClusterMaxNF = 4;
+struct ClusterPlan {
+    int nf, n_tiles, S, splits, top;
+    float fill;  // share of the GPU's CTA slots that the launch fills
+    size_t tile_bytes, tiles_bytes, extra_bytes, partial_bytes;  // tiles and partial sums: of one frequency
+    size_t total() const { return size_t(nf) * (tiles_bytes + partial_bytes) + extra_bytes; }
+};
+struct ClusterArgs {
+    int kind, normals, S, n_tiles, splits, top, nf;
+    int64_t n_src, n_tgt;
+    size_t tile_bytes;
+    PointsView src;
+    TgtView tgt;
+    double amp_scale;
+    TwoPiSplit tp;
+    const void* nodes;  // source clusters, by level
+    const void* boxes;  // target rectangles
+    StageGate* gate;
+    float gate_ratio;
+    int* status;
+    struct {
+        double k;
+        float kh, kl, kph, kpl;  // k and k / pi
+        uint8_t* tiles;
+        const double2* sigma;
+        double2* out;    // [splits][n_tgt] partial sums, or the field
+        double2* field;
+    } f[kClusterMaxNF];
+};
+// whether the clustered kernel takes stages of this kind and size, and its plan
+bool cluster_plan(int kind, int normals, int nf, int64_t n_src, int64_t n_tgt, int S, int splits, int max_auto_splits,
+                  ClusterPlan& p);
+// Prepares a stage in `base` (p.total() bytes, 256-byte aligned) and writes the
+// gate.  One frequency: the tiles are written in any case (the direct kernel
+// reads the same ones); several: only if the gate chooses the clustered kernel.
+int cluster_prepare(const rsi_stage& st, const double* ks, float gate_ratio, const PointsView& src, int64_t n_src,
+                    const double2* sigma, const TgtView& tgt, int64_t n_tgt, double2* field, const ClusterPlan& p,
+                    uint8_t* base, int* status, ClusterArgs& a, cudaStream_t s);
+// the sums and, where the sources are split, their reduction
+int cluster_run(const ClusterArgs& a, cudaStream_t s);
 int launch_stage_fp32(const StageArgs& a, cudaStream_t s);
 int launch_stage_fp64(const StageArgs& a, cudaStream_t s);
 int fp32_threads();
@@ -84,3 +172,6 @@ TimingScope timing_begin(cudaStream_t s);
 void timing_end(TimingScope& t, int kind, double pairs, cudaStream_t s);
 // out[j] = sum over splits of part[split][j] (Neumaier, split order)
 int launch_reduce_partials(const double2* part, int splits, int64_t n, double2* out, int* status, cudaStream_t s);
+// the same for the direct kernel beside the clustered one: nothing is done where the gate chose the other
+int launch_reduce_gated(const StageArgs& a, double2* out, cudaStream_t s);
+

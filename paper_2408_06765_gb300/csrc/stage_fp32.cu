@@ -11,6 +11,7 @@ template <int KIND, int NORM, int TPT, int VAR>
 __global__ void __launch_bounds__(kThreads, (min_blocks<KIND, TPT, VAR>()))
     stage_fp32_kernel(StageArgs a) {
     extern __shared__ __align__(128) uint8_t smem[];
+    if (a.gate && gate_clustered(a.gate, a.S, a.gate_ratio)) return;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + RSI_PIPE_STAGES * a.tile_bytes);
     init_barriers(bars);
     const int split = blockIdx.y;
@@ -35,7 +36,7 @@ __global__ void __launch_bounds__(kThreads, (min_blocks<KIND, TPT, VAR>()))
 __global__ void prep_fp32_kernel(int kind, int normals, int64_t n_src, PointsView src,
                                  const double2* __restrict__ sigma, double amp_scale, double k, uint8_t* tiles,
                                  size_t tile_bytes, int packed) {
-    __shared__ double red[32];
+    __shared__ __align__(8) float red[192];
     prep_tile(kind, normals, int(blockDim.x), n_src, src, sigma, amp_scale, k, tiles, tile_bytes,
               int64_t(blockIdx.x), red, packed != 0);
 }

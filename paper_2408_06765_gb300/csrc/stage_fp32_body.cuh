@@ -496,28 +496,113 @@ __device__ __forceinline__ double block_reduce(double v, bool is_max, double* sh
     return v;
 }
 
-// Writes tile `tile` (header + S records) of a source set; called by every
+// minima of six values over the CTA (every thread gets them); red: 6 x 32 floats.
+// FP32: this GPU's FP64 minima take 16 cycles a warp, and a tile needs hundreds
+__device__ __forceinline__ void block_min6(float (&v)[6], float* red) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+#pragma unroll
+    for (int d = 0; d < 6; ++d)
+#pragma unroll
+        for (int o = 16; o; o >>= 1) v[d] = fminf(v[d], __shfl_xor_sync(0xffffffffu, v[d], o));
+    __syncthreads();
+    if (lane == 0)
+#pragma unroll
+        for (int d = 0; d < 6; ++d) red[d * 32 + wid] = v[d];
+    __syncthreads();
+#pragma unroll
+    for (int d = 0; d < 6; ++d) {
+        v[d] = red[d * 32];
+        for (int q = 1; q < nw; ++q) v[d] = fminf(v[d], red[d * 32 + q]);
+    }
+}
+
+// Smallest and largest of three doubles over the CTA's threads with `use` (every
+// thread gets them; NaNs are passed over); red: 192 floats.  Compared as
+// integers of the same order: this GPU's FP64 pipe takes 16 cycles a warp.
+__device__ __forceinline__ void block_range3(const double (&x)[3], bool use, double (&lo)[3], double (&hi)[3],
+                                             float* red) {
+    const long long top = 0x7fffffffffffffffll;
+    long long* r = reinterpret_cast<long long*>(red);  // 3 x 32 at a time
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+        long long v[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            long long b = __double_as_longlong(side ? -x[d] : x[d]);
+            const bool nan = (b & top) > 0x7ff0000000000000ll;
+            b ^= (b >> 63) & top;  // as a signed integer in the doubles' order
+            v[d] = use && !nan ? b : top;
+#pragma unroll
+            for (int o = 16; o; o >>= 1) v[d] = min(v[d], __shfl_xor_sync(0xffffffffu, v[d], o));
+        }
+        __syncthreads();
+        if (lane == 0)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) r[d * 32 + wid] = v[d];
+        __syncthreads();
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            long long m = r[d * 32];
+            for (int q = 1; q < nw; ++q) m = min(m, r[d * 32 + q]);
+            m ^= (m >> 63) & top;
+            (side ? hi[d] : lo[d]) = side ? -__longlong_as_double(m) : __longlong_as_double(m);
+        }
+    }
+}
+
+// Slot of the i-th source in the order that tiles are cut in.  Mode 0: the
+// slots' own order, cells of (u, v) with as many cuts in u as in v.  Mode 1:
+// the cells of a disk or cap, where v is the angle: 8 sectors first, then cuts
+// in u and v in turn, so that a tile is about as long as it is wide (at 0.7 of
+// the radius the arc of an angle step is 2 pi times the radial step of the same
+// share).  Both are permutations of every aligned power-of-two block's slots.
+__device__ __forceinline__ int64_t source_slot(int64_t i, int64_t n, int mode) {
+    if (!mode) return i;
+    const int m = 63 - __clzll(static_cast<long long>(i ^ n));
+    const int64_t start = n & ~((int64_t(2) << m) - 1);
+    const uint32_t pos = uint32_t(i - start);
+    const int a = (m + 1) >> 1, b = m >> 1, lead = b >= 4 ? 3 : 0;
+    uint32_t out = 0;
+    int u = a - 1, v = b - 1, bit = m - 1;  // highest bits left
+    for (int q = 0; q < lead; ++q, --v, --bit) out |= ((pos >> bit) & 1u) << (2 * v + 1);
+    bool take_u = true;
+    for (; bit >= 0; --bit) {
+        const uint32_t x = (pos >> bit) & 1u;
+        if ((take_u && u >= 0) || v < 0) {
+            out |= x << (2 * u--);
+        } else {
+            out |= x << (2 * v-- + 1);
+        }
+        take_u = !take_u;
+    }
+    return start + int64_t(out);
+}
+
+// Writes tile `tile` (header + S records) of a source set (red: 192 floats of
+// shared memory); called by every
 // thread of a CTA of blockDim.x >= S threads (threads past S only take part
 // in the block reductions).
 __device__ __forceinline__ void prep_tile(int kind, int normals, int S, int64_t n_src, const PointsView& src,
                                           const double2* __restrict__ sigma, double amp_scale, double k,
-                                          uint8_t* tiles, size_t tile_bytes, int64_t tile, double* red,
-                                          bool packed = false) {
+                                          uint8_t* tiles, size_t tile_bytes, int64_t tile, float* red,
+                                          bool packed = false, int mode = 0) {
     const bool in_tile = int(threadIdx.x) < S;
-    const int64_t i = tile * S + threadIdx.x;
-    const bool valid = in_tile && i < n_src;
-    double c[3];
-    const double* coord[3] = {src.x, src.y, src.z};
-    for (int d = 0; d < 3; ++d) {
-        double v = valid ? coord[d][i] : 0.0;
-        double lo = block_reduce(valid ? v : INFINITY, false, red);
-        double hi = block_reduce(valid ? v : -INFINITY, true, red);
-        c[d] = 0.5 * (lo + hi);
-    }
+    const int64_t i0 = tile * S + threadIdx.x;
+    const bool valid = in_tile && i0 < n_src;
+    const int64_t i = valid ? source_slot(i0, n_src, mode) : i0;
+    // centre of the tile's box
     float ch[3], cl[3];
-    for (int d = 0; d < 3; ++d) {
-        ch[d] = __double2float_rn(c[d]);
-        cl[d] = __double2float_rn(c[d] - double(ch[d]));
+    {
+        double v[3] = {0.0, 0.0, 0.0}, lo[3], hi[3];
+        if (valid) v[0] = src.x[i], v[1] = src.y[i], v[2] = src.z[i];
+        block_range3(v, valid, lo, hi, red);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const double c = 0.5 * (lo[d] + hi[d]);
+            ch[d] = __double2float_rn(c);
+            cl[d] = __double2float_rn(c - double(ch[d]));
+        }
     }
     const int rec_f = (kind == RSI_STAGE_RSI && normals == RSI_NORMALS_POINTS) ? 12 : 8;
     float* rec = reinterpret_cast<float*>(tiles + size_t(tile) * tile_bytes + RSI_TILE_HDR_BYTES) +
@@ -592,7 +677,8 @@ __device__ __forceinline__ void prep_tile(int kind, int normals, int S, int64_t 
             rec[11 * fs] = -mag * fmaf(nx, px, fmaf(ny, py, nz * pz));  // -m n . p
         }
     }
-    double rad = block_reduce(double(radius2), true, red);
+    float rad[6] = {-radius2, 0.f, 0.f, 0.f, 0.f, 0.f};
+    block_min6(rad, red);
     if (threadIdx.x == 0) {
         float* hdr = reinterpret_cast<float*>(tiles + size_t(tile) * tile_bytes);
         hdr[0] = ch[0];
@@ -601,7 +687,7 @@ __device__ __forceinline__ void prep_tile(int kind, int normals, int S, int64_t 
         hdr[3] = cl[1];
         hdr[4] = ch[2];
         hdr[5] = cl[2];
-        hdr[6] = sqrtf(float(rad));
+        hdr[6] = sqrtf(-rad[0]);
         hdr[7] = 0.0f;
     }
 }

@@ -43,6 +43,9 @@ struct MultiArgs {
     // (double angle) instead of its own sincos
     int perm[kMaxNF];
     int harm;
+    // where the single-frequency clustered kernels are launched as well: the device's choice
+    const StageGate* gate;
+    float gate_ratio;
 };
 
 // Tile records (float4 units): [p.x, p.y, p.z, |p|^2], then
@@ -381,6 +384,7 @@ template <int KIND, int NORM, int NF, int PK, int HM>
 __global__ void __launch_bounds__(kThreads, PK ? (NF >= 4 ? 3 : HM ? RSI_MULTI_HARM_MIN_BLOCKS : RSI_MULTI_PACKED_MIN_BLOCKS) : 2)
     stage_multi_kernel(MultiArgs a) {
     extern __shared__ __align__(128) uint8_t smem[];
+    if (a.gate && gate_clustered(a.gate, a.S, a.gate_ratio)) return;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + RSI_PIPE_STAGES * a.tile_bytes);
     init_barriers(bars);
     constexpr int RF4 = mrec_f4<KIND, NORM, NF, PK>();  // float4 per record in the tiles
@@ -604,6 +608,7 @@ __global__ void mprep_kernel(int kind, int normals, int nf, int64_t n_src, Point
                              size_t tile_bytes) {
     __shared__ double red[32];
     const int S = blockDim.x;
+    if (a.gate && gate_clustered(a.gate, S, a.gate_ratio)) return;
     const int64_t tile = blockIdx.x;
     const int64_t i = tile * S + threadIdx.x;
     const bool valid = i < n_src;
@@ -767,6 +772,10 @@ struct MPlan {
     int S, n_tiles, tiles_per_split, splits;
     int64_t blocks;  // target blocks
     size_t tile_bytes, tiles_bytes, partial_bytes;
+    // the clustered kernel beside this one, its workspace after this one's
+    bool clustered;
+    ClusterPlan c;
+    size_t bytes() const { return tiles_bytes + partial_bytes + (clustered ? c.total() : 0); }
 };
 
 size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
@@ -856,6 +865,8 @@ int mplan(const rsi_stage& st, int nf, const double* ks, int64_t n_src, int64_t 
     p.blocks = blocks;
     a.tiles_per_split = p.tiles_per_split;
     a.splits = p.splits;
+    p.clustered = st.variant == 0 && !st.tile && !st.tpt &&
+                  cluster_plan(st.kind, st.normals, nf, n_src, n_tgt, p.S, st.splits, 128, p.c);
     return RSI_OK;
 }
 
@@ -867,7 +878,7 @@ extern "C" size_t rsi_stage_multi_workspace_bytes(const rsi_stage* st, int32_t n
     MPlan p;
     MultiArgs a = {};
     if (mplan(*st, nf, ks, n_src, n_tgt, p, a) != RSI_OK) return 0;
-    return p.tiles_bytes + p.partial_bytes;
+    return p.bytes();
 }
 
 extern "C" int rsi_propagate_stage_multi(const rsi_stage* st, int32_t nf, const double* ks, const void* src_points,
@@ -888,22 +899,39 @@ extern "C" int rsi_propagate_stage_multi(const rsi_stage* st, int32_t nf, const 
     MultiArgs a = {};
     int rc = mplan(*st, nf, ks, n_src, n_tgt, p, a);
     if (rc != RSI_OK) return rc;
-    if (workspace_bytes < p.tiles_bytes + p.partial_bytes)
+    if (workspace_bytes < p.bytes())
         return rsi_fail(RSI_E_NOMEM, "rsi_propagate_stage_multi: workspace %zu < %zu bytes", workspace_bytes,
-                        p.tiles_bytes + p.partial_bytes);
+                        p.bytes());
     int* status = rsi_status_ptr();
     if (!status) return RSI_E_CUDA;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     PointsView src = rsi_points_view(const_cast<void*>(src_points), n_src);
     PointsView tgt = rsi_points_view(const_cast<void*>(tgt_points), n_tgt);
     uint8_t* tiles = static_cast<uint8_t*>(workspace);
+    double2* field = reinterpret_cast<double2*>(tgt_field);
+    const TgtView tv = {tgt.xh, tgt.xl, tgt.yh, tgt.yl, tgt.zh, tgt.zl, tgt.x, tgt.y, tgt.z};
+    TimingScope tsc = {};
+    if (p.clustered) {
+        // every frequency through the clustered kernel, unless the device's
+        // estimate of all of them is in favour of the shared direct sum below,
+        // whose instructions per frequency are this share of a single stage's
+        const float ratio = nf == 2 ? 0.8f : a.harm ? 0.61f : nf == 3 ? 0.69f : 0.66f;
+        ClusterArgs c;
+        rc = cluster_prepare(*st, ks, ratio, src, n_src, reinterpret_cast<const double2*>(src_sigma), tv, n_tgt, field,
+                             p.c, tiles + p.tiles_bytes + p.partial_bytes, status, c, s);
+        if (rc != RSI_OK) return rc;
+        a.gate = c.gate;
+        a.gate_ratio = c.gate_ratio;
+        tsc = timing_begin(s);
+        rc = cluster_run(c, s);
+        if (rc != RSI_OK) return rc;
+    }
     mprep_kernel<<<p.n_tiles, p.S, 0, s>>>(a.kind, a.normals, nf, n_src, src,
                                            reinterpret_cast<const double2*>(src_sigma), stage_amp_scale(*st), a,
                                            tiles, p.tile_bytes);
     RSI_CHECK_LAUNCH("mprep_kernel");
     a.tiles = tiles;
-    a.tgt = {tgt.xh, tgt.xl, tgt.yh, tgt.yl, tgt.zh, tgt.zl, tgt.x, tgt.y, tgt.z};
-    double2* field = reinterpret_cast<double2*>(tgt_field);
+    a.tgt = tv;
     a.out = p.splits > 1 ? reinterpret_cast<double2*>(tiles + p.tiles_bytes) : field;
     a.field = field;
     a.done = nullptr;
@@ -914,7 +942,7 @@ extern "C" int rsi_propagate_stage_multi(const rsi_stage* st, int32_t nf, const 
                      "rsi_propagate_stage_multi: clear the completion counters");
     }
     a.status = status;
-    TimingScope tsc = timing_begin(s);
+    if (!p.clustered) tsc = timing_begin(s);
     int o = 0;
     rc = mdispatch(a, s, false, &o);
     if (rc != RSI_OK) return rc;

@@ -70,6 +70,11 @@ extern "C" int rsi_propagate_stage_noalloc(const rsi_stage* st, const void* src_
     rsi_stage s = *st;
     size_t need = rsi_stage_workspace_bytes(&s, n_src, n_tgt);
     if (need == 0) return RSI_E_INVAL;  // the stage description was rejected; message already set
+    if (need > kArea && s.precision == RSI_PREC_FP32C && s.variant == 0) {
+        // without room for the clustered kernel's tables the direct kernel (variant 3) runs
+        s.variant = 3;
+        need = rsi_stage_workspace_bytes(&s, n_src, n_tgt);
+    }
     if (need > kArea && s.splits == 0) {
         // The automatic split count wants more room for partial sums than the
         // static area has.  Each split holds n_tgt complex partial sums next to
