@@ -17,7 +17,7 @@
 // in the RSI stage kernel.
 #include <math.h>
 
-#include "stage.cuh"
+#include "stage_cluster_body.cuh"
 
 namespace {
 
@@ -53,6 +53,9 @@ struct RtArgs {
     TwoPiSplit tp;
     double2* out;            // [splits][n_tgt] partials, or the field
     int* status;
+    const StageGate* gate;   // where the clustered kernel is launched as well (null: this one runs)
+    float gate_ratio;
+    float k1p, k2p;          // k1 / pi, k2 / pi
 };
 
 // reference ray of one target through one tile centre
@@ -102,6 +105,9 @@ __device__ __forceinline__ void snell_residual(float t, float b, float h1q, floa
     m = fmaxf(r1, r2);
 }
 
+// FAST: the crossing's iteration ends when a step falls below 2^-21 of the
+// distance (the travel time is second order in it); else after 24 steps
+template <bool FAST = false>
 __device__ __forceinline__ RayRef ray_reference(float qxh, float qxl, float qyh, float qyl, float qzh, float qzl,
                                                 const float* c, const RtArgs& a) {
     RayRef R;
@@ -137,7 +143,10 @@ __device__ __forceinline__ RayRef ray_reference(float qxh, float qxl, float qyh,
         else
             lo = t;
         float tn = t - __fdividef(G, dG);
-        t = (tn >= lo && tn <= hi) ? tn : 0.5f * (lo + hi);
+        tn = (tn >= lo && tn <= hi) ? tn : 0.5f * (lo + hi);
+        const float step = fabsf(tn - t);
+        t = tn;
+        if (FAST && step <= 4.8e-7f * rh) break;
     }
     R.tc = t;
     // b = rho_c - t_c and the path lengths, as double-floats
@@ -305,9 +314,12 @@ __device__ __forceinline__ float2 sub2(float2 x, float2 y) { return __ffma2_rn(y
 // a negated per-tile constant or an FMA by -1 (no packed negations), the
 // reciprocal square roots, divisions, clamps and sincos per point, and the
 // safeguarded steps only for a point whose ray has not converged
+//
+// ray_core2: D1 - D1c and D2 - D2c, and T12 / sqrt(spreading) as the product
+// of tn and rs
 template <int NW>
-__device__ __forceinline__ void ray_pair2(const RayRef& R, float2 px, float2 py, float2 pzn, float2 A,
-                                          const RtArgs& a, float k1, float k2, float2& acc_r, float2& acc_i) {
+__device__ __forceinline__ void ray_core2(const RayRef& R, float2 px, float2 py, float2 pzn, const RtArgs& a,
+                                          float2& dD1, float2& dD2, float2& tn, float2& rs) {
     const float2 vx = sub2(f2(R.dx), px), vy = sub2(f2(R.dy), py);
     const float2 v2 = __ffma2_rn(vx, vx, __fmul2_rn(vy, vy));
     const bool okx = v2.x > 1e-24f, oky = v2.y > 1e-24f;
@@ -373,16 +385,25 @@ __device__ __forceinline__ void ray_pair2(const RayRef& R, float2 px, float2 py,
     // t - am (D + Dc) = am (-(D + Dc)) + t with -(D + Dc) = D (-1) - Dc
     const float2 am1 = __fadd2_rn(D1, f2(-R.D1)), am2 = __fadd2_rn(D2, f2(-R.D2));
     const float2 ns1 = __ffma2_rn(D1, f2(-1.0f), f2(-R.D1)), ns2 = __ffma2_rn(D2, f2(-1.0f), f2(-R.D2));
-    const float2 dD1 = __ffma2_rn(__ffma2_rn(am1, ns1, t1), __fmul2_rn(f2(0.5f), ir1), am1);
-    const float2 dD2 = __ffma2_rn(__ffma2_rn(am2, ns2, t2), __fmul2_rn(f2(0.5f), ir2), am2);
-    const float2 u = __ffma2_rn(f2(k1), dD1, __ffma2_rn(f2(k2), dD2, f2(R.tau)));
+    dD1 = __ffma2_rn(__ffma2_rn(am1, ns1, t1), __fmul2_rn(f2(0.5f), ir1), am1);
+    dD2 = __ffma2_rn(__ffma2_rn(am2, ns2, t2), __fmul2_rn(f2(0.5f), ir2), am2);
     const float2 cos1 = __fmul2_rn(h1, ir1), cos2 = __fmul2_rn(f2(h2), ir2);
-    const float2 tn = __fmul2_rn(f2(a.Tn), cos1), td = __ffma2_rn(f2(a.Td1), cos1, __fmul2_rn(f2(a.Td2), cos2));
+    tn = __fmul2_rn(f2(a.Tn), cos1);
+    const float2 td = __ffma2_rn(f2(a.Td1), cos1, __fmul2_rn(f2(a.Td2), cos2));
     // T12 = tn / td folded into the spreading's reciprocal square root, as in ray_pair
     const float2 cc = __fmul2_rn(__fmul2_rn(__fmul2_rn(f2(a.c21), cos1), cos1), f2(R.ih22));
     const float2 den = __fmul2_rn(__ffma2_rn(cc, __fmul2_rn(D2, q2), D1), __ffma2_rn(f2(a.c21), D2, D1));
     const float2 dt2 = __fmul2_rn(den, __fmul2_rn(td, td));
-    const float2 amp = __fmul2_rn(__fmul2_rn(A, tn), make_float2(rsqrt_ap(dt2.x), rsqrt_ap(dt2.y)));
+    rs = make_float2(rsqrt_ap(dt2.x), rsqrt_ap(dt2.y));
+}
+
+template <int NW>
+__device__ __forceinline__ void ray_pair2(const RayRef& R, float2 px, float2 py, float2 pzn, float2 A,
+                                          const RtArgs& a, float k1, float k2, float2& acc_r, float2& acc_i) {
+    float2 dD1, dD2, tn, rs;
+    ray_core2<NW>(R, px, py, pzn, a, dD1, dD2, tn, rs);
+    const float2 u = __ffma2_rn(f2(k1), dD1, __ffma2_rn(f2(k2), dD2, f2(R.tau)));
+    const float2 amp = __fmul2_rn(__fmul2_rn(A, tn), rs);
     float2 sn, cs;
     __sincosf(u.x, &sn.x, &cs.x);
     __sincosf(u.y, &sn.y, &cs.y);
@@ -400,6 +421,7 @@ __device__ __forceinline__ void ray_pair2(const RayRef& R, float2 px, float2 py,
 template <int TPT, int NW>
 __global__ void __launch_bounds__(kRtThreads, RSI_RT_MIN_BLOCKS) raytrace_kernel(RtArgs a) {
     extern __shared__ __align__(128) uint8_t smem[];
+    if (a.gate && gate_clustered(a.gate, a.S, a.gate_ratio)) return;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + RSI_PIPE_STAGES * a.tile_bytes);
     const int tid = threadIdx.x;
     if (tid == 0) {
@@ -513,6 +535,269 @@ __global__ void __launch_bounds__(kRtThreads, RSI_RT_MIN_BLOCKS) raytrace_kernel
     }
 }
 
+// ---------------------------------------------------------------------------
+// The clustered sum (stage_cluster_body.cuh) over refracted rays: with Psi(p, q)
+// = k1 D1 + k2 D2 of the ray from c + p to b + q,
+//   Psi(p, q) = Psi(p, 0) + Psi(0, q) - Psi(0, 0) + k delta(p, q),
+// and e^{ik delta} T12 / sqrt(spreading) is interpolated on the nodes.  A pair
+// of a 4096-point cluster and a 1024-target block at 10 nodes per axis takes
+// some 60 000 instructions a warp in place of 16 million.
+// ---------------------------------------------------------------------------
+struct RayModel {
+    static constexpr bool kPolar = false;
+    static constexpr int kDirectCost = 976;  // 122 instructions per pair (ncu), 256 targets over 32 lanes
+    using Ref = RayRef;
+    const rsi_cluster::Sum& g;
+    const RtArgs& a;
+
+    // As choose_nodes, with the cross derivatives of Psi: K_r along the line of
+    // the feet (the tilts of the ray turn vertical offsets into horizontal ones),
+    // K_t across it.  sep adds to the clusters' size over the ray's length (in
+    // the slower medium's wavelengths) the change of the slowness over what is
+    // left of it to grazing.  The lines phi(sep) of choose_nodes hold: errors
+    // over random tilted pistons and depths of 0.5 to 58 mm below 5e-7.
+    __device__ __forceinline__ int choose(const rsi_cluster::Node& s, const rsi_cluster::Box& b) const {
+        if (!(s.flat > 0.0f) || b.q3 != 0.0f) return 0;
+        float dx, dy, h1, h2, lo;
+        df_diff(b.c[0], b.c[1], s.c[0], s.c[1], dx, lo);
+        df_diff(b.c[2], b.c[3], s.c[2], s.c[3], dy, lo);
+        df_diff(a.zIh, a.zIl, s.c[4], s.c[5], h1, lo);
+        df_diff(b.c[4], b.c[5], a.zIh, a.zIl, h2, lo);
+        const float hd = sqrtf(fmaf(s.h1, s.h1, s.h2 * s.h2)), qd = sqrtf(fmaf(b.q1, b.q1, b.q2 * b.q2));
+        if (!(h1 > hd) || !(h2 > (b.ax2 == 2 ? b.q2 : 0.0f))) return 0;
+        const float rho = sqrtf(fmaf(dx, dx, dy * dy));
+        const float h1q = h1 * h1, h2q = h2 * h2;
+        float lo_t = 0.0f, hi_t = rho, t = rho * __fdividef(h1, fmaf(a.c21, h2, h1));
+#pragma unroll 1
+        for (int it = 0; it < 16; ++it) {
+            float G, dG, m;
+            snell_residual(t, rho - t, h1q, h2q, a.s1, a.s2, a.s1 * h1q, a.s2 * h2q, G, dG, m);
+            (G > 0.0f ? hi_t : lo_t) = t;
+            float tn = t - __fdividef(G, dG);
+            tn = (tn >= lo_t && tn <= hi_t) ? tn : 0.5f * (lo_t + hi_t);
+            const bool end = fabsf(tn - t) <= 1e-5f * rho;
+            t = tn;
+            if (end) break;
+        }
+        const float D1 = sqrtf(fmaf(t, t, h1q)), D2 = sqrtf(fmaf(rho - t, rho - t, h2q));
+        const float s1 = t / D1, c1 = h1 / D1, s2 = (rho - t) / D2, c2 = h2 / D2, t1 = s1 / c1, t2 = s2 / c2;
+        const float ik1 = 1.0f / a.k1h, ik2 = 1.0f / a.k2h;
+        const float w1 = ik1 / (c1 * c1), w2 = ik2 / (c2 * c2);
+        const float Kt = 1.0f / fmaf(D1, ik1, D2 * ik2), Kr = 1.0f / fmaf(D1, w1, D2 * w2);
+        const float ux = rho > 0.0f ? dx / rho : 1.0f, uy = rho > 0.0f ? dy / rho : 0.0f;
+        const float sep = (hd + qd) * Kt * fmaxf(ik1, ik2) + Kr * (hd / c1 + qd / c2) * fmaxf(s1 * w1, s2 * w2);
+        // the effective offsets along and across the line of the feet
+        const float e1r = fmaf(s.e1[0], ux, fmaf(s.e1[1], uy, -t1 * s.e1[2])), e1t = fmaf(s.e1[1], ux, -s.e1[0] * uy);
+        const float e2r = fmaf(s.e2[0], ux, fmaf(s.e2[1], uy, -t1 * s.e2[2])), e2t = fmaf(s.e2[1], ux, -s.e2[0] * uy);
+        const float v1r = b.ax1 == 0 ? ux : uy, v1t = b.ax1 == 0 ? -uy : ux;
+        const float v2r = b.ax2 == 1 ? uy : -t2, v2t = b.ax2 == 1 ? ux : 0.0f;
+        const float m11 = fabsf(fmaf(Kr * e1r, v1r, Kt * e1t * v1t)) * s.h1 * b.q1;
+        const float m12 = fabsf(fmaf(Kr * e1r, v2r, Kt * e1t * v2t)) * s.h1 * b.q2;
+        const float m21 = fabsf(fmaf(Kr * e2r, v1r, Kt * e2t * v1t)) * s.h2 * b.q1;
+        const float m22 = fabsf(fmaf(Kr * e2r, v2r, Kt * e2t * v2t)) * s.h2 * b.q2;
+        if (!((fmaxf(Kr, Kt) * qd / c2 + 1.0f / D1) * s.h3 <= 5e-7f)) return 0;  // sources off the rectangle's plane
+        const float phi = fmaxf(fmaxf(m11 + m12, m21 + m22), fmaxf(m11 + m21, m12 + m22)) + Kt * hd * qd * sep;
+        return rsi_cluster::nodes_for(phi, sep);
+    }
+    __device__ __forceinline__ static float cost(float ns, float nt, int N) {
+        return rsi_cluster::pair_cost(ns, nt, N, 130.f, 480.f, 180.f);
+    }
+    __device__ __forceinline__ Ref reference(const float* t, const float* c) const {
+        return ray_reference<true>(t[0], t[1], t[2], t[3], t[4], t[5], c, a);
+    }
+    __device__ __forceinline__ Ref broadcast(const Ref& r, int lane) const {
+        constexpr int n = sizeof(Ref) / sizeof(float);
+        Ref o;
+        const float* from = reinterpret_cast<const float*>(&r);
+        float* to = reinterpret_cast<float*>(&o);
+#pragma unroll
+        for (int i = 0; i < n; ++i) to[i] = __shfl_sync(0xffffffffu, from[i], lane);
+        return o;
+    }
+    __device__ __forceinline__ float2 source_phase(const Ref& r, float2 px, float2 py, float2 pzn, float2) const {
+        float2 dD1, dD2, tn, rs;
+        ray_core2<1>(r, px, py, pzn, a, dD1, dD2, tn, rs);
+        return __ffma2_rn(f2(a.k1p), dD1, __ffma2_rn(f2(a.k2p), dD2, f2(0.318309886f * r.tau)));
+    }
+    __device__ __forceinline__ void prepare_targets(rsi_cluster::WarpArea&, const rsi_cluster::Box&,
+                                                    const rsi_cluster::Box&) const {}
+    __device__ __forceinline__ void centre_phase(const rsi_cluster::WarpArea&, const rsi_cluster::Box&,
+                                                 const rsi_cluster::Box&, const Ref& r, float& c, float& s) const {
+        sincospif(0.318309886f * r.tau, &s, &c);
+    }
+    __device__ __forceinline__ void target(const rsi_cluster::WarpArea& w, const rsi_cluster::TargetPos&, int j,
+                                           float& c, float& s) const {
+        const Ref r = ray_reference<true>(__ldg(a.tgt.xh + j), __ldg(a.tgt.xl + j), __ldg(a.tgt.yh + j),
+                                          __ldg(a.tgt.yl + j), __ldg(a.tgt.zh + j), __ldg(a.tgt.zl + j), w.node.c, a);
+        sincospif(0.318309886f * r.tau, &s, &c);
+    }
+    // record: px, py, -pz, -(Psi(p, 0) - Psi(0, 0)), beta, m
+    __device__ __forceinline__ void node_record(const rsi_cluster::Box&, const Ref& r, const float3& p, float m,
+                                                float beta, float* q) const {
+        float2 dD1, dD2, tn, rs;
+        ray_core2<1>(r, f2(p.x), f2(p.y), f2(-p.z), a, dD1, dD2, tn, rs);
+        q[0] = p.x;
+        q[2] = p.y;
+        q[4] = -p.z;
+        q[6] = -fmaf(a.k1h, dD1.x, a.k2h * dD2.x);
+        q[8] = beta;
+        q[10] = m;
+        q[12] = q[14] = 0.0f;
+    }
+    __device__ __forceinline__ float2 node_field(const rsi_cluster::Node& s, const rsi_cluster::Box& b, const Ref&,
+                                                 float q1, float q2, const float4* pr, int i0, int i1) const {
+        float t[6];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const float o = d == b.ax1 ? q1 : d == b.ax2 ? q2 : 0.0f;
+            df_diff(b.c[2 * d], b.c[2 * d + 1], -o, 0.0f, t[2 * d], t[2 * d + 1]);
+        }
+        const Ref r = ray_reference<true>(t[0], t[1], t[2], t[3], t[4], t[5], s.c, a);
+        float2 ar = f2(0.0f), ai = f2(0.0f);
+#pragma unroll 1
+        for (int i = i0; i < i1; ++i) {
+            const float4 v0 = pr[4 * i], v1 = pr[4 * i + 1], v2 = pr[4 * i + 2];
+            float2 dD1, dD2, tn, rs, sn, cs;
+            ray_core2<1>(r, make_float2(v0.x, v0.y), make_float2(v0.z, v0.w), make_float2(v1.x, v1.y), a, dD1, dD2, tn, rs);
+            const float2 dl = __fadd2_rn(__ffma2_rn(f2(a.k1h), dD1, __fmul2_rn(f2(a.k2h), dD2)), make_float2(v1.z, v1.w));
+            const float2 u = __fadd2_rn(dl, make_float2(v2.x, v2.y));
+            __sincosf(u.x, &sn.x, &cs.x);
+            __sincosf(u.y, &sn.y, &cs.y);
+            const float2 amp = __fmul2_rn(__fmul2_rn(make_float2(v2.z, v2.w), tn), rs);
+            ar = __ffma2_rn(amp, cs, ar);
+            ai = __ffma2_rn(amp, sn, ai);
+        }
+        return make_float2(ar.x + ar.y, ai.x + ai.y);
+    }
+    __device__ __forceinline__ float2 direct(const float* hdr, const float4* rec, int64_t j) const {
+        const Ref r = ray_reference(__ldg(a.tgt.xh + j), __ldg(a.tgt.xl + j), __ldg(a.tgt.yh + j),
+                                    __ldg(a.tgt.yl + j), __ldg(a.tgt.zh + j), __ldg(a.tgt.zl + j), hdr, a);
+        float2 pr = f2(0.0f), pi = f2(0.0f);
+#pragma unroll 1
+        for (int i = 0; i < a.S; i += 2) {
+            const float4 v0 = rec[2 * i], v1 = rec[2 * i + 1], v2 = rec[2 * i + 2];
+            ray_pair2<1>(r, make_float2(v0.x, v0.y), make_float2(v0.z, v0.w), make_float2(v1.x, v1.y),
+                         make_float2(v2.x, v2.y), a, a.k1h, a.k2h, pr, pi);
+        }
+        return make_float2(pr.x + pr.y, pi.x + pi.y);
+    }
+};
+
+constexpr int kClTpt = 4;  // a block: 1024 targets
+struct RtClusterArgs {
+    RtArgs a;  // splits: the clustered kernel's; out: its partial sums [splits + segs][n_tgt]
+    int top, segs;
+    float weight;
+    uint8_t* left;
+    int* any;
+    int64_t n_src;
+    PointsView src;
+    double amp_scale, k;
+    uint8_t* tiles;
+    rsi_cluster::Node* nodes;
+    rsi_cluster::Box* boxes;
+    StageGate* gate;
+    double2* field;
+};
+
+__device__ __forceinline__ rsi_cluster::Sum cluster_sum(const RtClusterArgs& c) {
+    rsi_cluster::Sum g = {};
+    g.tiles = c.tiles;
+    g.tile_bytes = uint32_t(c.a.tile_bytes);
+    g.S = c.a.S;
+    g.rec_f = 8;
+    g.n_tiles = c.a.n_tiles;
+    g.nodes[0] = c.nodes;
+    g.nodes[1] = c.nodes + c.a.n_tiles;
+    g.nodes[2] = g.nodes[1] + (c.a.n_tiles + 3) / 4;
+    g.boxes = c.boxes;
+    g.top = c.top;
+    g.tgt = c.a.tgt;
+    g.n_tgt = c.a.n_tgt;
+    g.status = c.a.status;
+    return g;
+}
+
+__global__ void __launch_bounds__(rsi_cluster::kThreads, 2)
+    raytrace_cluster_kernel(const __grid_constant__ RtClusterArgs c) {
+    using namespace rsi_cluster;
+    extern __shared__ __align__(128) uint8_t smem[];
+    if (!gate_clustered(c.gate, c.a.S, c.a.gate_ratio)) return;
+    Shared& sh = *reinterpret_cast<Shared*>(smem);
+    float4* acc = reinterpret_cast<float4*>(smem + sizeof(Shared));
+    int* slot = reinterpret_cast<int*>(acc + kClTpt * kThreads);
+    init_shared(sh);
+    const Sum g = cluster_sum(c);
+    run_block<RayModel, kClTpt>(RayModel{g, c.a}, g, int64_t(blockIdx.x) * kClTpt * kThreads, blockIdx.y, c.a.splits,
+                                c.gate->L, c.gate->h, c.a.out + size_t(blockIdx.y) * size_t(c.a.n_tgt),
+                                c.left + size_t(blockIdx.x) * size_t(c.a.n_tiles), c.any + blockIdx.x, sh, acc, slot);
+}
+
+__global__ void __launch_bounds__(rsi_cluster::kThreads, RSI_RT_MIN_BLOCKS)
+    raytrace_leftover_kernel(const __grid_constant__ RtClusterArgs c) {
+    extern __shared__ __align__(128) uint8_t smem[];
+    const int block = blockIdx.x / kClTpt;
+    if (!gate_clustered(c.gate, c.a.S, c.a.gate_ratio) || !c.any[block]) return;
+    const rsi_cluster::Sum g = cluster_sum(c);
+    rsi_cluster::leftover_block<RayModel, kClTpt>(RayModel{g, c.a}, g, block, blockIdx.x % kClTpt, blockIdx.y, c.segs,
+                                                  c.gate->L, c.gate->h, c.left + size_t(block) * size_t(c.a.n_tiles),
+                                                  c.a.out + size_t(c.a.splits + blockIdx.y) * size_t(c.a.n_tgt), smem);
+}
+
+// tiles and their clusters, the larger clusters, the rectangles of the targets
+__global__ void __launch_bounds__(rsi_cluster::kThreads)
+    raytrace_prep_kernel(const __grid_constant__ RtClusterArgs c) {
+    using namespace rsi_cluster;
+    __shared__ __align__(8) float red[192];
+    int b = blockIdx.x;
+    const int n_tiles = c.a.n_tiles, groups = (n_tiles + 3) / 4, clusters = n_tiles + groups + (groups + 3) / 4;
+    if (b >= clusters) {
+        b -= clusters;
+        int L, h;
+        find_rows(c.a.tgt, c.a.n_tgt, kClTpt * kThreads, L, h);
+        make_boxes<kClTpt>(c.a.tgt, c.a.n_tgt, int64_t(b) * kClTpt * kThreads, L, h, c.boxes + 5 * int64_t(b), red);
+        if (b == 0 && threadIdx.x == 0) *c.gate = StageGate{L, h, 0, 0};
+        if (threadIdx.x == 0) c.any[b] = 0;
+        return;
+    }
+    b = clusters - 1 - b;  // the large clusters, which take longest, first
+    const int mode = source_mode(RSI_STAGE_PISTON, c.src, c.n_src, red);
+    if (b < n_tiles)
+        rsi_fp32::prep_tile(RSI_STAGE_PISTON, RSI_NORMALS_Z, c.a.S, c.n_src, c.src, nullptr, c.amp_scale, c.k, c.tiles,
+                            c.a.tile_bytes, b, red, true, mode);
+    Node* nodes = c.nodes;
+    int64_t len = c.a.S;
+    int count = n_tiles;
+    for (int l = 0; l < kLevels; ++l) {
+        if (b < count) {
+            const int64_t i0 = b * len, i1 = i0 + len < c.n_src ? i0 + len : c.n_src;
+            make_node(RSI_STAGE_PISTON, RSI_NORMALS_Z, c.src, c.n_src, mode, i0, i1, nodes + b, red);
+            return;
+        }
+        b -= count;
+        nodes += count;
+        count = (count + 3) / 4;
+        len *= 4;
+    }
+}
+
+__global__ void raytrace_estimate_kernel(const __grid_constant__ RtClusterArgs c, int blocks) {
+    const int b = int(int64_t(blockIdx.x) * blocks / gridDim.x);
+    const rsi_cluster::Sum g = {};
+    rsi_cluster::estimate<RayModel, kClTpt>(RayModel{g, c.a}, c.nodes, c.a.n_tiles, c.a.S, c.top, c.boxes + 5 * int64_t(b),
+                                            c.weight, blockIdx.x, c.gate);
+}
+
+__global__ void raytrace_reduce_kernel(const __grid_constant__ RtClusterArgs c, const double2* __restrict__ direct,
+                                       int direct_splits) {
+    const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (gate_clustered(c.gate, c.a.S, c.a.gate_ratio))
+        rsi_cluster::sum_block_order<kClTpt>(c.a.out, c.a.splits, c.segs, c.any, t, c.a.n_tgt, c.gate->L, c.gate->h,
+                                             c.field, c.a.status);
+    else if (direct_splits > 1 && t < c.a.n_tgt)
+        sum_partials(direct + t, direct_splits, c.a.n_tgt, c.field + t, c.a.status);
+}
+
 constexpr int kTpt = 1;
 
 size_t rt_smem(size_t tile_bytes) { return RSI_PIPE_STAGES * tile_bytes + RSI_PIPE_STAGES * sizeof(uint64_t); }
@@ -520,6 +805,12 @@ size_t rt_smem(size_t tile_bytes) { return RSI_PIPE_STAGES * tile_bytes + RSI_PI
 struct RtPlan {
     int S, n_tiles, tiles_per_split, splits;
     size_t tile_bytes, tiles_bytes, partial_bytes;
+    // the clustered kernel beside the direct one: the same kernel plan as a
+    // piston stage's (ClusterPlan), its partial sums before the direct one's
+    bool clustered;
+    ClusterPlan c;
+    size_t part_at() const { return clustered ? c.total() : tiles_bytes; }
+    size_t bytes() const { return part_at() + partial_bytes; }
 };
 
 size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
@@ -570,6 +861,8 @@ int rt_plan(const rsi_raytrace& rt, int64_t n_src, int64_t n_tgt, RtPlan& p) {
     p.tiles_per_split = (p.n_tiles + splits - 1) / splits;
     p.splits = (p.n_tiles + p.tiles_per_split - 1) / p.tiles_per_split;
     p.partial_bytes = p.splits > 1 ? align256(size_t(p.splits) * size_t(n_tgt) * sizeof(double2)) : 0;
+    p.clustered = !rt.tile && !rt.newton &&
+                  cluster_plan(RSI_TIMING_RAYTRACE, RSI_NORMALS_Z, 1, n_src, n_tgt, p.S, rt.splits, 128, p.c);
     return RSI_OK;
 }
 
@@ -598,7 +891,7 @@ extern "C" size_t rsi_raytrace_workspace_bytes(const rsi_raytrace* rt, int64_t n
     if (!rt) return 0;
     RtPlan p;
     if (rt_plan(*rt, n_src, n_tgt, p) != RSI_OK) return 0;
-    return p.tiles_bytes + p.partial_bytes;
+    return p.bytes();
 }
 
 extern "C" int rsi_raytrace_field(const rsi_raytrace* rt, const void* src_points, int64_t n_src,
@@ -612,9 +905,8 @@ extern "C" int rsi_raytrace_field(const rsi_raytrace* rt, const void* src_points
     RtPlan p;
     int rc = rt_plan(*rt, n_src, n_tgt, p);
     if (rc != RSI_OK) return rc;
-    if (workspace_bytes < p.tiles_bytes + p.partial_bytes)
-        return rsi_fail(RSI_E_NOMEM, "rsi_raytrace_field: workspace %zu < %zu bytes", workspace_bytes,
-                        p.tiles_bytes + p.partial_bytes);
+    if (workspace_bytes < p.bytes())
+        return rsi_fail(RSI_E_NOMEM, "rsi_raytrace_field: workspace %zu < %zu bytes", workspace_bytes, p.bytes());
     int* status = rsi_status_ptr();
     if (!status) return RSI_E_CUDA;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -626,9 +918,6 @@ extern "C" int rsi_raytrace_field(const rsi_raytrace* rt, const void* src_points
     st.precision = RSI_PREC_FP32C;
     st.k = rt->k1;
     st.v0 = rt->v0;
-    rc = launch_prep_fp32(st, src, n_src, nullptr, p.S, tiles, p.tile_bytes, p.n_tiles, s, RSI_RT_PACKED != 0);
-    if (rc != RSI_OK) return rc;
-
     RtArgs a = {};
     a.tiles = tiles;
     a.tile_bytes = p.tile_bytes;
@@ -651,10 +940,59 @@ extern "C" int rsi_raytrace_field(const rsi_raytrace* rt, const void* src_points
     a.newton = rt->newton ? rt->newton : 1;
     a.tp = two_pi_split();
     double2* field = reinterpret_cast<double2*>(tgt_field);
-    a.out = p.splits > 1 ? reinterpret_cast<double2*>(tiles + p.tiles_bytes) : field;
+    double2* part = reinterpret_cast<double2*>(tiles + p.part_at());
+    a.out = p.splits > 1 ? part : field;
     a.status = status;
+    a.k1p = float(rt->k1 / M_PI);
+    a.k2p = float(rt->k2 / M_PI);
+    RtClusterArgs c;
+    if (p.clustered) {
+        c.n_src = n_src;
+        c.src = src;
+        c.amp_scale = stage_amp_scale(st);
+        c.k = st.k;
+        c.top = p.c.top;
+        c.tiles = tiles;
+        uint8_t* extra = tiles + p.c.tiles_bytes;
+        c.nodes = reinterpret_cast<rsi_cluster::Node*>(extra);
+        c.boxes = reinterpret_cast<rsi_cluster::Box*>(extra + p.c.boxes_at);
+        c.gate = reinterpret_cast<StageGate*>(extra + p.c.extra_bytes - 256);
+        c.field = field;
+        a.gate = c.gate;
+        a.gate_ratio = float(RayModel::kDirectCost) / 134.4f;
+        c.weight = kClusterWeight / p.c.fill;
+        c.a = a;
+        c.a.splits = p.c.splits;
+        c.a.out = reinterpret_cast<double2*>(extra + p.c.extra_bytes);
+        c.segs = p.c.segs;
+        c.left = extra + p.c.left_at;
+        c.any = reinterpret_cast<int*>(extra + p.c.any_at);
+        const int groups = (p.n_tiles + 3) / 4, roots = (groups + 3) / 4, blocks = int((n_tgt + 1023) / 1024);
+        raytrace_prep_kernel<<<unsigned(p.n_tiles + groups + roots + blocks), rsi_cluster::kThreads, 0, s>>>(c);
+        RSI_CHECK_LAUNCH("raytrace_prep_kernel");
+        raytrace_estimate_kernel<<<16, rsi_cluster::kThreads, 0, s>>>(c, blocks);
+        RSI_CHECK_LAUNCH("raytrace_estimate_kernel");
+    } else {
+        rc = launch_prep_fp32(st, src, n_src, nullptr, p.S, tiles, p.tile_bytes, p.n_tiles, s, RSI_RT_PACKED != 0);
+        if (rc != RSI_OK) return rc;
+    }
 
     TimingScope tsc = timing_begin(s);
+    if (p.clustered) {
+        constexpr size_t smem = rsi_cluster::smem_bytes<kClTpt>();
+        static RsiCtxOnce attr;
+        if (attr.needed()) {
+            RSI_CUDA_TRY(cudaFuncSetAttribute(raytrace_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem),
+                         "cudaFuncSetAttribute(raytrace_cluster)");
+            attr.done();
+        }
+        raytrace_cluster_kernel<<<dim3(unsigned((n_tgt + 1023) / 1024), unsigned(p.c.splits)), rsi_cluster::kThreads,
+                                  smem, s>>>(c);
+        RSI_CHECK_LAUNCH("raytrace_cluster_kernel");
+        raytrace_leftover_kernel<<<dim3(unsigned((n_tgt + 1023) / 1024 * kClTpt), unsigned(p.c.segs)),
+                                   rsi_cluster::kThreads, rsi_cluster::leftover_smem(p.tile_bytes), s>>>(c);
+        RSI_CHECK_LAUNCH("raytrace_leftover_kernel");
+    }
     const int64_t per_block = int64_t(kRtThreads) * kTpt;
     dim3 grid(unsigned((n_tgt + per_block - 1) / per_block), unsigned(p.splits));
     switch (a.newton) {  // the common step counts unrolled
@@ -665,6 +1003,11 @@ extern "C" int rsi_raytrace_field(const rsi_raytrace* rt, const void* src_points
     }
     if (rc != RSI_OK) return rc;
     timing_end(tsc, RSI_TIMING_RAYTRACE, double(n_src) * double(n_tgt), s);
+    if (p.clustered) {
+        raytrace_reduce_kernel<<<unsigned((n_tgt + 1023) / 1024 * 4), 256, 0, s>>>(c, part, p.splits);
+        RSI_CHECK_LAUNCH("raytrace_reduce_kernel");
+        return RSI_OK;
+    }
     if (p.splits > 1) return launch_reduce_partials(a.out, p.splits, n_tgt, field, status, s);
     return RSI_OK;
 }

@@ -93,10 +93,13 @@ namespace {
 
 __global__ void reduce_partials_kernel(const double2* __restrict__ part, int splits, int64_t n,
                                        double2* __restrict__ out, int* status) {
-    reduce_partials(part, splits, n, out, status);
+    const int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (j < n) sum_partials(part + j, splits, n, out + j, status);
 }
 __global__ void reduce_gated_kernel(StageArgs a, double2* __restrict__ out) {
-    if (!gate_clustered(a.gate, a.S, a.gate_ratio)) reduce_partials(a.out, a.splits, a.n_tgt, out, a.status);
+    const int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (j < a.n_tgt && !gate_clustered(a.gate, a.S, a.gate_ratio))
+        sum_partials(a.out + j, a.splits, a.n_tgt, out + j, a.status);
 }
 
 size_t align256(size_t v) { return (v + 255) & ~size_t(255); }

@@ -35,30 +35,26 @@ TwoPiSplit two_pi_split();
 // preparation, stage_cluster_body.cuh)
 struct StageGate {
     int L, h;                  // rows of the target set and strip height of the block order
-    unsigned long long cost;   // estimated instructions of the clustered kernel over the sampled pairs
+    unsigned long long cost;   // estimated weighted instructions of the clustered kernel over the sampled pairs
     unsigned long long pairs;  // samples: a tile and a quarter block (256 targets) each
 };
-// Which of the two kernels runs: the clustered kernel's estimated instructions
-// per warp, over all the stage's frequencies, against the direct sum's (16.8
-// per 32 pairs, 256 S pairs), which issues them 1.5 times as fast.  `ratio`: a
-// multi-frequency stage's instructions per frequency over a single stage's,
-// times the share of the GPU that the clustered kernel's CTAs fill.  On a
-// laminate's stages 0.5 mm apart, where the estimate is 0.6 of the direct sum's
-// instructions and 0.84 of the GPU is filled, both take 3.1 ms (2^16 x 2^16, 5
-// MHz).  FP32 arithmetic on integers: the same in every thread of both kernels.
+// Which of the two kernels runs.  `cost`: the instructions per warp that the
+// clustered kernel would take, over all the stage's frequencies, weighted by how
+// much slower it issues them than the direct kernel (estimate()), and those of
+// the direct sums it leaves; against the direct kernel's 16.8 per 32 pairs, 256
+// S pairs per sample.  `ratio`: a multi-frequency stage's instructions per
+// frequency, or a ray's per pair, over a single stage's.  FP32 arithmetic on
+// integers: the same in every thread of both kernels.
 __device__ __forceinline__ bool gate_clustered(const StageGate* g, int S, float ratio) {
-    return float(g->cost) * 1.5f < float(g->pairs) * (134.4f * float(S)) * ratio;
+    return float(g->cost) * 1.05f < float(g->pairs) * (134.4f * float(S)) * ratio;
 }
 
-// out[j] = sum over splits of part[split][j], j = this thread
-__device__ __forceinline__ void reduce_partials(const double2* __restrict__ part, int splits, int64_t n,
-                                                double2* __restrict__ out, int* status) {
-    int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (j >= n) return;
-    // Neumaier summation over the splits in index order
+// *out = sum of part[0], part[stride], ... (n terms; Neumaier, FP64, in order)
+__device__ __forceinline__ void sum_partials(const double2* __restrict__ part, int n, int64_t stride, double2* out,
+                                             int* status) {
     double sr = 0.0, cr = 0.0, si = 0.0, ci = 0.0;
-    for (int s = 0; s < splits; ++s) {
-        double2 v = part[size_t(s) * size_t(n) + size_t(j)];
+    for (int s = 0; s < n; ++s) {
+        double2 v = part[size_t(s) * size_t(stride)];
         double t = sr + v.x;
         cr += (fabs(sr) >= fabs(v.x)) ? (sr - t) + v.x : (v.x - t) + sr;
         sr = t;
@@ -68,7 +64,7 @@ __device__ __forceinline__ void reduce_partials(const double2* __restrict__ part
     }
     double re = sr + cr, im = si + ci;
     if (!isfinite(re) || !isfinite(im)) atomicExch(status, RSI_DEV_NONFINITE);
-    out[j] = make_double2(re, im);
+    *out = make_double2(re, im);
 }
 
 struct StageArgs {
@@ -116,14 +112,17 @@ int launch_prep_fp64(const rsi_stage& st, const PointsView& src, int64_t n_src, 
 // clusters and the rectangles of the targets, the gate last), then per
 // frequency the partial sums.
 constexpr int kClusterMaxNF = 4;
+constexpr float kClusterWeight = 1.5f;  // issue rate of the direct kernel (0.75 and more) over the clustered one's (0.5)
 struct ClusterPlan {
     int nf, n_tiles, S, splits, top;
+    int segs;    // CTAs per quarter block for the leftovers
     float fill;  // share of the GPU's CTA slots that the launch fills
     size_t tile_bytes, tiles_bytes, extra_bytes, partial_bytes;  // tiles and partial sums: of one frequency
+    size_t boxes_at, left_at, any_at;  // within extra
     size_t total() const { return size_t(nf) * (tiles_bytes + partial_bytes) + extra_bytes; }
 };
 struct ClusterArgs {
-    int kind, normals, S, n_tiles, splits, top, nf;
+    int kind, normals, S, n_tiles, splits, segs, top, nf;
     int64_t n_src, n_tgt;
     size_t tile_bytes;
     PointsView src;
@@ -133,18 +132,21 @@ struct ClusterArgs {
     const void* nodes;  // source clusters, by level
     const void* boxes;  // target rectangles
     StageGate* gate;
-    float gate_ratio;
+    float gate_ratio, weight;
     int* status;
     struct {
         double k;
         float kh, kl, kph, kpl;  // k and k / pi
         uint8_t* tiles;
         const double2* sigma;
-        double2* out;    // [splits][n_tgt] partial sums, or the field
+        double2* part;   // [splits + segs][n_tgt]
         double2* field;
+        uint8_t* left;   // [blocks][n_tiles] quarters left to the direct sum
+        int* any;        // [blocks] whether there are some
     } f[kClusterMaxNF];
 };
-// whether the clustered kernel takes stages of this kind and size, and its plan
+// whether the clustered kernel takes stages of this kind (RSI_TIMING_RAYTRACE: the
+// ray-tracing sum) and size, and its plan
 bool cluster_plan(int kind, int normals, int nf, int64_t n_src, int64_t n_tgt, int S, int splits, int max_auto_splits,
                   ClusterPlan& p);
 // Prepares a stage in `base` (p.total() bytes, 256-byte aligned) and writes the

@@ -14,16 +14,8 @@ using namespace rsi_cluster;
 
 constexpr int kTpt = 4;  // a block: 1024 targets
 
-template <int KIND, int NORM>
-__global__ void __launch_bounds__(kThreads, 2) cluster_kernel(const __grid_constant__ ClusterArgs a) {
-    extern __shared__ __align__(128) uint8_t smem[];
-    Shared& sh = *reinterpret_cast<Shared*>(smem);
-    float4* acc = reinterpret_cast<float4*>(smem + sizeof(Shared));
-    int* slot = reinterpret_cast<int*>(acc + kTpt * kThreads);
-    uint64_t* bars = reinterpret_cast<uint64_t*>(slot + kTpt * kThreads);
-    if (!gate_clustered(a.gate, a.S, a.gate_ratio)) return;
-    init_shared(sh, bars);
-    const auto& f = a.f[blockIdx.z];
+__device__ __forceinline__ Sum stage_sum(const ClusterArgs& a, int fi) {
+    const auto& f = a.f[fi];
     Sum g;
     g.tiles = f.tiles;
     g.tile_bytes = uint32_t(a.tile_bytes);
@@ -44,15 +36,46 @@ __global__ void __launch_bounds__(kThreads, 2) cluster_kernel(const __grid_const
     g.kpl = f.kpl;
     g.tp = a.tp;
     g.status = a.status;
-    double2* out = f.out + (a.splits > 1 ? size_t(blockIdx.y) * size_t(a.n_tgt) : 0);
-    uint32_t uses = 0;
-    run_block<KIND, NORM, kTpt>(g, int64_t(blockIdx.x) * kTpt * kThreads, blockIdx.y, a.splits, a.gate->L, a.gate->h,
-                                out, sh, acc, slot, bars, uses);
+    return g;
+}
+
+// CTA (block, split, frequency)
+template <int KIND, int NORM>
+__global__ void __launch_bounds__(kThreads, 2) cluster_kernel(const __grid_constant__ ClusterArgs a) {
+    extern __shared__ __align__(128) uint8_t smem[];
+    Shared& sh = *reinterpret_cast<Shared*>(smem);
+    float4* acc = reinterpret_cast<float4*>(smem + sizeof(Shared));
+    int* slot = reinterpret_cast<int*>(acc + kTpt * kThreads);
+    if (!gate_clustered(a.gate, a.S, a.gate_ratio)) return;
+    init_shared(sh);
+    const Sum g = stage_sum(a, blockIdx.z);
+    const auto& f = a.f[blockIdx.z];
+    run_block<StageModel<KIND, NORM>, kTpt>(StageModel<KIND, NORM>{g}, g, int64_t(blockIdx.x) * kTpt * kThreads,
+                                            blockIdx.y, a.splits, a.gate->L, a.gate->h,
+                                            f.part + size_t(blockIdx.y) * size_t(a.n_tgt),
+                                            f.left + size_t(blockIdx.x) * size_t(a.n_tiles), f.any + blockIdx.x, sh, acc,
+                                            slot);
+}
+
+// CTA (quarter block, segment, frequency)
+template <int KIND, int NORM>
+__global__ void __launch_bounds__(kThreads, 4) leftover_kernel(const __grid_constant__ ClusterArgs a) {
+    extern __shared__ __align__(128) uint8_t smem[];
+    const auto& f = a.f[blockIdx.z];
+    const int block = blockIdx.x / kTpt;
+    if (!gate_clustered(a.gate, a.S, a.gate_ratio) || !f.any[block]) return;
+    const Sum g = stage_sum(a, blockIdx.z);
+    leftover_block<StageModel<KIND, NORM>, kTpt>(StageModel<KIND, NORM>{g}, g, block, blockIdx.x % kTpt, blockIdx.y,
+                                                 a.segs, a.gate->L, a.gate->h,
+                                                 f.left + size_t(block) * size_t(a.n_tiles),
+                                                 f.part + size_t(a.splits + blockIdx.y) * size_t(a.n_tgt), smem);
 }
 
 __global__ void cluster_reduce_kernel(const __grid_constant__ ClusterArgs a) {
+    const auto& f = a.f[blockIdx.y];
     if (gate_clustered(a.gate, a.S, a.gate_ratio))
-        reduce_partials(a.f[blockIdx.y].out, a.splits, a.n_tgt, a.f[blockIdx.y].field, a.status);
+        sum_block_order<kTpt>(f.part, a.splits, a.segs, f.any, int64_t(blockIdx.x) * blockDim.x + threadIdx.x, a.n_tgt,
+                              a.gate->L, a.gate->h, f.field, a.status);
 }
 
 // CTAs 0 .. n_tiles - 1: a tile (if `tiles`) and its cluster each; then the
@@ -69,8 +92,10 @@ __global__ void __launch_bounds__(kThreads) cluster_prep_kernel(const __grid_con
         Box* boxes = static_cast<Box*>(const_cast<void*>(a.boxes));
         make_boxes<kTpt>(a.tgt, a.n_tgt, int64_t(b) * kTpt * kThreads, L, h, boxes + 5 * int64_t(b), red);
         if (b == 0 && threadIdx.x == 0) *a.gate = StageGate{L, h, 0, 0};
+        if (int(threadIdx.x) < a.nf) a.f[threadIdx.x].any[b] = 0;
         return;
     }
+    b = clusters - 1 - b;  // the large clusters, which take longest, first
     const int mode = source_mode(a.kind, a.src, a.n_src, red);
     if (b < a.n_tiles && tiles)
         rsi_fp32::prep_tile(a.kind, a.normals, a.S, a.n_src, a.src, a.f[0].sigma, a.amp_scale, a.f[0].k, a.f[0].tiles,
@@ -103,8 +128,11 @@ constexpr int kEstimates = 16;  // CTAs of the cost estimate, per frequency
 
 __global__ void cluster_estimate_kernel(const __grid_constant__ ClusterArgs a, int blocks) {
     const int b = int(int64_t(blockIdx.x) * blocks / gridDim.x);
-    estimate<kTpt>(static_cast<const Node*>(a.nodes), a.n_tiles, a.S, a.top,
-                   static_cast<const Box*>(a.boxes) + 5 * int64_t(b), a.f[blockIdx.y].kh, blockIdx.x, a.gate);
+    Sum g = {};
+    g.kh = a.f[blockIdx.y].kh;
+    using Model = StageModel<RSI_STAGE_PISTON, RSI_NORMALS_Z>;  // both kinds choose and cost alike
+    estimate<Model, kTpt>(Model{g}, static_cast<const Node*>(a.nodes), a.n_tiles, a.S, a.top,
+                          static_cast<const Box*>(a.boxes) + 5 * int64_t(b), a.weight, blockIdx.x, a.gate);
 }
 
 int64_t target_blocks(int64_t n_tgt) { return (n_tgt + kTpt * kThreads - 1) / (kTpt * kThreads); }
@@ -124,14 +152,18 @@ int run_t(const ClusterArgs* a, cudaStream_t s, int* occ) {
             *occ = 1;
         return RSI_OK;
     }
-    dim3 grid(unsigned(target_blocks(a->n_tgt)), unsigned(a->splits), unsigned(a->nf));
-    kern<<<grid, kThreads, smem, s>>>(*a);
+    const unsigned blocks = unsigned(target_blocks(a->n_tgt));
+    kern<<<dim3(blocks, unsigned(a->splits), unsigned(a->nf)), kThreads, smem, s>>>(*a);
     RSI_CHECK_LAUNCH("cluster_kernel");
+    leftover_kernel<KIND, NORM><<<dim3(blocks * kTpt, unsigned(a->segs), unsigned(a->nf)), kThreads,
+                                  leftover_smem(a->tile_bytes), s>>>(*a);
+    RSI_CHECK_LAUNCH("leftover_kernel");
     return RSI_OK;
 }
 
 int dispatch(int kind, const ClusterArgs* a, cudaStream_t s, int* occ) {
-    return kind == RSI_STAGE_PISTON ? run_t<RSI_STAGE_PISTON, RSI_NORMALS_Z>(a, s, occ)
+    // (the ray-tracing sum's kernel has the same shared memory and registers as the piston's)
+    return kind != RSI_STAGE_RSI ? run_t<RSI_STAGE_PISTON, RSI_NORMALS_Z>(a, s, occ)
                                     : run_t<RSI_STAGE_RSI, RSI_NORMALS_Z>(a, s, occ);
 }
 
@@ -147,14 +179,16 @@ size_t nodes_bytes(int n_tiles) {
 // more than the direct kernel's preparation, and 4e8 pairs take that kernel
 // 0.3 ms.  A piston's clusters are small beside the distance and nearly always
 // taken; an interface's may not be, so its sums have to be longer, and those of
-// several frequencies, whose direct sum is shared, twice as long.  Per-point normals turn within a
+// several frequencies, whose direct sum is shared, twice as long; a ray costs the
+// direct kernel 6 times a stage's pair.  Per-point normals turn within a
 // tile on every curved surface, where the direct sum would be taken anyway.
 bool cluster_plan(int kind, int normals, int nf, int64_t n_src, int64_t n_tgt, int S, int splits, int max_auto_splits,
                   ClusterPlan& p) {
-    const double least = (kind == RSI_STAGE_PISTON ? 4e8 : 1e9) * (nf > 1 ? 2.0 : 1.0);
+    const double least = kind == RSI_TIMING_RAYTRACE ? 3e8 : (kind == RSI_STAGE_PISTON ? 4e8 : 1e9) * (nf > 1 ? 2.0 : 1.0);
     if (n_src < 8192 || n_tgt < 4096 || double(n_src) * double(n_tgt) < least) return false;
-    if (kind != RSI_STAGE_PISTON && base_normals(normals) != RSI_NORMALS_Z) return false;
+    if (kind == RSI_STAGE_RSI && base_normals(normals) != RSI_NORMALS_Z) return false;
     const int n_tiles = int((n_src + S - 1) / S);
+    if (n_tiles >= 1 << 22) return false;  // an item's tile index has 22 bits
     const int64_t blocks = target_blocks(n_tgt);
     const int64_t roots = (n_tiles + kRootTiles - 1) / kRootTiles;
     // A batch takes 8 pairs of clusters at once: with fewer than 6 roots a CTA
@@ -190,8 +224,15 @@ bool cluster_plan(int kind, int normals, int nf, int64_t n_src, int64_t n_tgt, i
     p.fill = float(std::min(1.0, double(blocks * p.splits * nf) / double(slots)));
     p.tile_bytes = RSI_TILE_HDR_BYTES + size_t(S) * fp32_record_bytes(kind, base_normals(normals));
     p.tiles_bytes = align256(size_t(n_tiles) * p.tile_bytes);
-    p.extra_bytes = nodes_bytes(n_tiles) + align256(size_t(blocks) * 5 * sizeof(Box)) + 256;
-    p.partial_bytes = p.splits > 1 ? align256(size_t(p.splits) * size_t(n_tgt) * sizeof(double2)) : 0;
+    p.boxes_at = nodes_bytes(n_tiles);
+    p.left_at = p.boxes_at + align256(size_t(blocks) * 5 * sizeof(Box));
+    p.any_at = p.left_at + align256(size_t(nf) * size_t(blocks) * size_t(n_tiles));
+    p.extra_bytes = p.any_at + align256(size_t(nf) * size_t(blocks) * sizeof(int)) + 256;
+    // 16 segments: a block next to the sources is left whole, and its four
+    // quarters are then 64 CTAs' work; fewer where the sum has blocks enough
+    // (at most 2^24 partial sums)
+    p.segs = int(std::max<int64_t>(1, std::min<int64_t>({16, n_tiles / 4, (int64_t(1) << 24) / n_tgt})));
+    p.partial_bytes = align256(size_t(p.splits + p.segs) * size_t(n_tgt) * sizeof(double2));
     return true;
 }
 
@@ -204,6 +245,7 @@ int cluster_prepare(const rsi_stage& st, const double* ks, float gate_ratio, con
     a.S = p.S;
     a.n_tiles = p.n_tiles;
     a.splits = p.splits;
+    a.segs = p.segs;
     a.top = p.top;
     a.nf = p.nf;
     a.n_src = n_src;
@@ -215,9 +257,10 @@ int cluster_prepare(const rsi_stage& st, const double* ks, float gate_ratio, con
     a.tp = two_pi_split();
     uint8_t* extra = base + size_t(p.nf) * p.tiles_bytes;
     a.nodes = extra;
-    a.boxes = extra + nodes_bytes(p.n_tiles);
+    a.boxes = extra + p.boxes_at;
     a.gate = reinterpret_cast<StageGate*>(extra + p.extra_bytes - 256);
-    a.gate_ratio = gate_ratio * p.fill;
+    a.gate_ratio = gate_ratio;
+    a.weight = kClusterWeight / p.fill;
     a.status = status;
     for (int f = 0; f < p.nf; ++f) {
         auto& q = a.f[f];
@@ -229,7 +272,9 @@ int cluster_prepare(const rsi_stage& st, const double* ks, float gate_ratio, con
         q.tiles = base + size_t(f) * p.tiles_bytes;
         q.sigma = sigma ? sigma + size_t(f) * size_t(n_src) : nullptr;
         q.field = field + size_t(f) * size_t(n_tgt);
-        q.out = p.splits > 1 ? reinterpret_cast<double2*>(extra + p.extra_bytes + size_t(f) * p.partial_bytes) : q.field;
+        q.part = reinterpret_cast<double2*>(extra + p.extra_bytes + size_t(f) * p.partial_bytes);
+        q.left = extra + p.left_at + size_t(f) * size_t(target_blocks(n_tgt)) * size_t(p.n_tiles);
+        q.any = reinterpret_cast<int*>(extra + p.any_at) + size_t(f) * size_t(target_blocks(n_tgt));
     }
     const int groups = (p.n_tiles + 3) / 4, roots = (groups + 3) / 4;
     const unsigned blocks = unsigned(target_blocks(n_tgt));
@@ -246,8 +291,8 @@ int cluster_prepare(const rsi_stage& st, const double* ks, float gate_ratio, con
 
 int cluster_run(const ClusterArgs& a, cudaStream_t s) {
     const int rc = dispatch(a.kind, &a, s, nullptr);
-    if (rc != RSI_OK || a.splits == 1) return rc;
-    cluster_reduce_kernel<<<dim3(unsigned((a.n_tgt + 255) / 256), unsigned(a.nf)), 256, 0, s>>>(a);
+    if (rc != RSI_OK) return rc;
+    cluster_reduce_kernel<<<dim3(unsigned(target_blocks(a.n_tgt) * kTpt), unsigned(a.nf)), 256, 0, s>>>(a);
     RSI_CHECK_LAUNCH("cluster_reduce_kernel");
     return RSI_OK;
 }

@@ -86,7 +86,6 @@ struct Shared {
     float tab[kTabFloats];
     Box box[5];
     int items[kRound * 4];
-    int direct[kRound];
     int warp_sum[kWarps];
 };
 
@@ -97,7 +96,7 @@ __device__ __forceinline__ int make_item(int n, int box, int level, int tile) {
 
 template <int TPT>
 constexpr size_t smem_bytes() {
-    return sizeof(Shared) + TPT * kThreads * (sizeof(float4) + sizeof(int)) + 2 * sizeof(uint64_t);
+    return sizeof(Shared) + TPT * kThreads * (sizeof(float4) + sizeof(int));
 }
 
 // Slot of the t-th target of the block order.  A set of n targets in rows of
@@ -124,14 +123,23 @@ __device__ __forceinline__ int block_pos(int i, int h) {
     return (i & 512) | (((i & 255) >> (b - 1)) << b) | (((i >> 8) & 1) << (b - 1)) | (i & lo);
 }
 
+// Nodes per axis for a phase excursion phi and a relative size sep.  The lines
+// phi(sep) were fitted to the largest error over random pairs of rectangles
+// (tilts, shapes and directions): below about 5e-7 of the term's magnitude,
+// 5e-8 root mean square, against 5e-7 to 1e-6 of FP32 rounding per pair term.
+__device__ __forceinline__ int nodes_for(float phi, float sep) {
+    if (sep <= 0.25f && phi <= 0.45f - 1.5f * sep) return 6;
+    if (sep <= 0.28f && phi <= 1.15f - 1.8f * sep) return 8;
+    if (sep <= 0.36f && phi <= 2.0f - 2.0f * sep) return 10;
+    if (sep <= 0.42f && phi <= 3.0f - 2.0f * sep) return 12;
+    return 0;
+}
+
 // Nodes per axis for a source cluster and a target cluster, 0 if they are not
 // admitted.  phi bounds the phase k delta that one axis of either rectangle
 // sees: its bilinear part (k / R) (u_a . v_b - (u_a . d/R)(v_b . d/R)) h_a q_b
 // summed over the other rectangle's axes, plus the cubic terms' size; sep is
-// the two rectangles' half diagonals over R.  The lines phi(sep) were fitted
-// to the largest error over random pairs of rectangles (tilts, shapes and
-// directions): below about 5e-7 of the term's magnitude, 5e-8 root mean
-// square, against 5e-7 to 1e-6 of FP32 rounding per pair term.
+// the two rectangles' half diagonals over R.
 __device__ __forceinline__ int choose_nodes(const Node& s, const Box& b, float k) {
     if (!(s.flat > 0.0f) || b.q3 != 0.0f) return 0;
     float d[3], lo;
@@ -142,10 +150,7 @@ __device__ __forceinline__ int choose_nodes(const Node& s, const Box& b, float k
     if (!(R > 0.0f)) return 0;
     const float iR = 1.0f / R;
     const float hd = sqrtf(s.h1 * s.h1 + s.h2 * s.h2), qd = sqrtf(b.q1 * b.q1 + b.q2 * b.q2);
-#ifndef RSI_CL_SEP
-#define RSI_CL_SEP 1.0f
-#endif
-    const float sep = RSI_CL_SEP * (hd + qd) * iR;
+    const float sep = (hd + qd) * iR;
     // what the rectangle leaves out: sources off its plane
     if (!((k * qd + 1.0f) * s.h3 * iR <= 5e-7f)) return 0;
     const float d1 = (d[0] * s.e1[0] + d[1] * s.e1[1] + d[2] * s.e1[2]) * iR;
@@ -156,15 +161,8 @@ __device__ __forceinline__ int choose_nodes(const Node& s, const Box& b, float k
     const float f = k * iR;
     const float m11 = f * fabsf(u11 - d1 * v1) * s.h1 * b.q1, m12 = f * fabsf(u12 - d1 * v2) * s.h1 * b.q2;
     const float m21 = f * fabsf(u21 - d2 * v1) * s.h2 * b.q1, m22 = f * fabsf(u22 - d2 * v2) * s.h2 * b.q2;
-    float phi = fmaxf(fmaxf(m11 + m12, m21 + m22), fmaxf(m11 + m21, m12 + m22)) + f * hd * qd * sep;
-#ifdef RSI_CL_PHI
-    phi *= RSI_CL_PHI;
-#endif
-    if (sep <= 0.25f && phi <= 0.45f - 1.5f * sep) return 6;
-    if (sep <= 0.28f && phi <= 1.15f - 1.8f * sep) return 8;
-    if (sep <= 0.36f && phi <= 2.0f - 2.0f * sep) return 10;
-    if (sep <= 0.42f && phi <= 3.0f - 2.0f * sep) return 12;
-    return 0;
+    const float phi = fmaxf(fmaxf(m11 + m12, m21 + m22), fmaxf(m11 + m21, m12 + m22)) + f * hd * qd * sep;
+    return nodes_for(phi, sep);
 }
 
 // |d - p| - R for an offset p: th = (|d - p|^2 - R^2) / 2, one Newton step
@@ -184,14 +182,15 @@ struct NodeRef {
 };
 
 // Instructions per warp that a pair of a source cluster of `ns` sources and a
-// target cluster of `nt` targets takes with N x N nodes (counted in the code),
-// and that the direct sum takes (16.8 per 32 pairs, measured)
-__device__ __forceinline__ float pair_cost(float ns, float nt, int N) {
+// target cluster of `nt` targets takes with N x N nodes: `src` of them for 64
+// sources' phases, `node` for two source nodes onto 32 target nodes, `tgt` for
+// 32 targets beside the interpolation (counted in the code)
+__device__ __forceinline__ float pair_cost(float ns, float nt, int N, float node, float tgt, float src) {
     const float n = float(N), nn = n * n;
-    const float src = 150.0f + ns * (1.2f + (4.0f + 2.5f * n) * (1.0f / 64.0f) * (32 / (32 / N)));
-    const float node = (N == 6 ? 3.0f : ceilf(nn * (1.0f / 32.0f))) * (60.0f + 18.0f * nn * (N == 6 ? 0.5f : 1.0f));
-    const float tgt = nt * (1.0f / 32.0f) * (85.0f + 1.5f * nn + 4.0f * n);
-    return src + node + tgt + 4.0f * ceilf(nn * (1.0f / 32.0f)) * (3.0f * n + 15.0f);
+    const float rounds = N == 6 ? 3.0f : ceilf(nn * (1.0f / 32.0f)), pairs = N == 6 ? 9.0f : 0.5f * nn;
+    return 150.0f + ns * (1.0f / 64.0f) * (src + (4.0f + 2.5f * n) * (32 / (32 / N))) +
+           rounds * (1.7f * node + node * pairs) + nt * (1.0f / 32.0f) * (tgt + 1.5f * nn + 4.0f * n) +
+           4.0f * ceilf(nn * (1.0f / 32.0f)) * (3.0f * n + 15.0f);
 }
 
 // Two source nodes onto one target node.  Records (pair-interleaved):
@@ -231,6 +230,8 @@ __device__ __forceinline__ void node_pair2(const NodeRef& n, const float4& v0, c
         b2 = __ffma2_rn(g, cs, b2);
     }
 }
+
+__device__ __forceinline__ float2 dup(float v) { return make_float2(v, v); }
 
 struct Sum {
     const uint8_t* tiles;
@@ -297,8 +298,6 @@ constexpr int node_groups() {
     return N == 6 ? 2 : 1;
 }
 
-__device__ __forceinline__ float2 dup(float v) { return make_float2(v, v); }
-
 // U_0 .. U_{N-1} of two points, pair-interleaved
 template <int N>
 __device__ __forceinline__ void cheb_row(float2 x, float* row) {
@@ -315,9 +314,9 @@ __device__ __forceinline__ void cheb_row(float2 x, float* row) {
 // One warp: moments of a source cluster for a target cluster, the field at the
 // target nodes and its Chebyshev coefficients (w.fh), the phase of the target
 // (e^{ik |Q_j - c|}, c the source cluster's centre) left out.
-template <int KIND, int N>
-__device__ __forceinline__ void warp_item(const Sum& g, const Box& b, const Box& b0, int t0, int nt, WarpArea& w,
-                                          const float* tab) {
+template <class M, int N>
+__device__ __forceinline__ void warp_item(const M& model, const Sum& g, const Box& b, const Box& b0, int t0, int nt,
+                                          WarpArea& w, const float* tab) {
     constexpr int NN = N * N, STR = 4 * N + 4;  // row stride: 16-byte groups without bank conflicts
     static_assert(32 * STR <= kRowFloats && NN * 8 <= kRowFloats, "warp area");
     constexpr int G = 32 / N;  // source groups of the product
@@ -325,9 +324,8 @@ __device__ __forceinline__ void warp_item(const Sum& g, const Box& b, const Box&
     const int lane = threadIdx.x & 31;
     const float* C = tab + tab_off(N);
     const Node& s = w.node;
-    const float k = g.kh;
     // references of the target cluster's centre: lanes 0 .. 15 the tiles, 16 the cluster
-    rsi_fp32::TgtRef ref;
+    typename M::Ref ref;
     float gx = 0.f, gy = 0.f, gz = 0.f;  // tile centre - cluster centre
     {
         const float* hc = lane < 16 ? reinterpret_cast<const float*>(g.tiles + size_t(t0 + min(lane, nt - 1)) * g.tile_bytes)
@@ -335,7 +333,7 @@ __device__ __forceinline__ void warp_item(const Sum& g, const Box& b, const Box&
         float c[6];
 #pragma unroll
         for (int q = 0; q < 6; ++q) c[q] = hc[q];
-        ref = rsi_fp32::target_reference(b.c[0], b.c[1], b.c[2], b.c[3], b.c[4], b.c[5], c, g.kh, g.kl, g.tp);
+        ref = model.reference(b.c, c);
         float lo;
         df_diff(c[0], c[1], s.c[0], s.c[1], gx, lo);
         df_diff(c[2], c[3], s.c[2], s.c[3], gy, lo);
@@ -352,13 +350,9 @@ __device__ __forceinline__ void warp_item(const Sum& g, const Box& b, const Box&
         for (int q = 0; q < 2 * N; q += 2) *reinterpret_cast<float2*>(part_m + q) = make_float2(0.f, 0.f);
     // -- moments: a lane takes a pair of sources in packed arithmetic, then one
     // column l of the product over every G-th pair
-    const float2 k2 = dup(k);
-    const float2 magic = dup(12582912.0f), nmagic = dup(-12582912.0f);  // 1.5 2^23: rounds to an integer
 #pragma unroll 1
     for (int t = 0; t < nt; ++t) {
-        const float Dx = __shfl_sync(0xffffffffu, ref.Dx, t), Dy = __shfl_sync(0xffffffffu, ref.Dy, t),
-                    Dz = __shfl_sync(0xffffffffu, ref.Dz, t), R = __shfl_sync(0xffffffffu, ref.R, t),
-                    tau = 0.318309886f * __shfl_sync(0xffffffffu, ref.tau, t);
+        const typename M::Ref rt = model.broadcast(ref, t);
         const float tx = __shfl_sync(0xffffffffu, gx, t), ty = __shfl_sync(0xffffffffu, gy, t),
                     tz = __shfl_sync(0xffffffffu, gz, t);
         const float o1 = fmaf(tx, f1.x, fmaf(ty, f1.y, tz * f1.z)), o2 = fmaf(tx, f2.x, fmaf(ty, f2.y, tz * f2.z));
@@ -372,20 +366,10 @@ __device__ __forceinline__ void warp_item(const Sum& g, const Box& b, const Box&
             const float4* r = reinterpret_cast<const float4*>(tile) + min(pi, (g.S >> 1) - 1) * (g.rec_f >> 1);
             const float4 v0 = __ldg(r), v1 = __ldg(r + 1), v2 = __ldg(r + 2);
             const float2 px = make_float2(v0.x, v0.y), py = make_float2(v0.z, v0.w), pzn = make_float2(v1.x, v1.y);
-            float2 m = KIND == RSI_STAGE_PISTON ? make_float2(v2.x, v2.y) : make_float2(v2.z, v2.w);
+            float2 m = M::kPolar ? make_float2(v2.z, v2.w) : make_float2(v2.x, v2.y);
             if (pi >= (g.S >> 1)) m = make_float2(0.f, 0.f);
-            const float2 th = __ffma2_rn(dup(-Dx), px, __ffma2_rn(dup(-Dy), py, __ffma2_rn(dup(Dz), pzn, make_float2(v1.z, v1.w))));
-            const float2 r2 = __ffma2_rn(th, dup(2.0f), dup(R * R));
-            const float2 ir = make_float2(rsqrt_approx(r2.x), rsqrt_approx(r2.y));
-            const float2 r0 = __fmul2_rn(r2, ir);
-            const float2 am = __fadd2_rn(r0, dup(-R));
-            const float2 a = __ffma2_rn(__ffma2_rn(am, __ffma2_rn(r0, dup(-0.5f), dup(-0.5f * R)), th), ir, am);
-            // the phase k (|d - c_tile| + a) + beta in half turns
-            const float2 ph = __fmul2_rn(dup(g.kph), a);
-            const float2 pl = __ffma2_rn(dup(g.kpl), a, __ffma2_rn(dup(g.kph), a, __fmul2_rn(dup(-g.kph), a)));
-            const float2 x = __ffma2_rn(__fadd2_rn(__ffma2_rn(ph, dup(0.5f), magic), nmagic), dup(-2.0f), ph);
-            float2 u = __fadd2_rn(x, __fadd2_rn(pl, dup(tau)));
-            if (KIND != RSI_STAGE_PISTON) u = __ffma2_rn(make_float2(v2.x, v2.y), dup(0.318309886f), u);
+            float2 u = model.source_phase(rt, px, py, pzn, make_float2(v1.z, v1.w));  // half turns
+            if (M::kPolar) u = __ffma2_rn(make_float2(v2.x, v2.y), dup(0.318309886f), u);
             float2 sn, cs;
             sincospif(u.x, &sn.x, &cs.x);
             sincospif(u.y, &sn.y, &cs.y);
@@ -452,105 +436,37 @@ __device__ __forceinline__ void warp_item(const Sum& g, const Box& b, const Box&
         w.y[o] = y;
     }
     __syncwarp();
-    // the cluster's own reference
-    const float Dx = __shfl_sync(0xffffffffu, ref.Dx, 16), Dy = __shfl_sync(0xffffffffu, ref.Dy, 16),
-                Dz = __shfl_sync(0xffffffffu, ref.Dz, 16), R = __shfl_sync(0xffffffffu, ref.R, 16);
-    const float R2 = R * R;
-    const bool x1 = b.ax1 == 0, y2 = b.ax2 == 1;
-    if (lane == 0) {  // for the targets' phases: the block's centre from the cluster's, exactly
-        float dh[3], dl[3], sh[3], sl[3];
-        for (int q = 0; q < 3; ++q) {
-            df_diff(b0.c[2 * q], b0.c[2 * q + 1], s.c[2 * q], s.c[2 * q + 1], dh[q], dl[q]);
-            df_sqr(dh[q], dl[q], sh[q], sl[q]);
-        }
-        df_add_pos(sh[0], sl[0], sh[1], sl[1], sh[0], sl[0]);
-        df_add_pos(sh[0], sl[0], sh[2], sl[2], w.S0h, w.S0l);
-        w.D1h = x1 ? dh[0] : dh[1], w.D1l = x1 ? dl[0] : dl[1];
-        w.D2h = y2 ? dh[1] : dh[2], w.D2l = y2 ? dl[1] : dl[2];
-    }
+    const typename M::Ref rc = model.broadcast(ref, 16);  // the cluster's own reference
+    model.prepare_targets(w, b, b0);
     __syncwarp();
-    float c0, s0;  // e^{ik |d|}, d the target cluster's centre from the source cluster's
-    {
-        TargetPos t;
-        df_diff(b.c[2 * b.ax1], b.c[2 * b.ax1 + 1], b0.c[2 * b.ax1], b0.c[2 * b.ax1 + 1], t.q1h, t.q1l);
-        df_diff(b.c[2 * b.ax2], b.c[2 * b.ax2 + 1], b0.c[2 * b.ax2], b0.c[2 * b.ax2 + 1], t.q2h, t.q2l);
-        float a1, e1, a2, e2;
-        df_sqr(t.q1h, t.q1l, a1, e1);
-        df_sqr(t.q2h, t.q2l, a2, e2);
-        df_add_pos(a1, e1, a2, e2, t.sh, t.sl);
-        target_phase(w, t, g.kph, g.kpl, c0, s0);
-    }
+    float c0, s0;  // the phase factor from the source cluster's centre to the target cluster's
+    model.centre_phase(w, b, b0, rc, c0, s0);
     for (int o = lane; o < NN; o += 32) {  // source node (a, c): moment and record
         const int a = o / N, c = o - a * N;
         float2 m2 = make_float2(0.f, 0.f);
 #pragma unroll
-        for (int q = 0; q < N; ++q) {
-            const float cc = C[c * N + q];
-            m2 = __ffma2_rn(make_float2(cc, cc), w.y[a * N + q], m2);
-        }
+        for (int q = 0; q < N; ++q) m2 = __ffma2_rn(dup(C[c * N + q]), w.y[a * N + q], m2);
         const float s1 = 0.5f * N * C[a * N + 1] * s.h1, s2 = 0.5f * N * C[c * N + 1] * s.h2;  // C[.][1] = (2/N) x_a
-        const float px = fmaf(s1, s.e1[0], s2 * s.e2[0]), py = fmaf(s1, s.e1[1], s2 * s.e2[1]),
-                    pz = fmaf(s1, s.e1[2], s2 * s.e2[2]);
-        const float t = fmaf(-Dx, px, fmaf(-Dy, py, fmaf(-Dz, pz, 0.5f * fmaf(px, px, fmaf(py, py, pz * pz)))));
-        // a = |d - p| - |d| for this t as a sum of two floats: r0 - R is exact, the Newton correction small
-        const float r2 = fmaf(2.0f, t, R2), ir = rsqrt_approx(r2), r0 = r2 * ir, am = r0 - R;
-        const float lo = fmaf(am, -0.5f * (r0 + R), t) * ir;
-        float mr = m2.x, mi = m2.y;
-        float m = sqrtf(fmaf(mr, mr, mi * mi));
-        // m e^{i beta} with arg in [-pi/2, pi/2]: a negated moment negates m alone
-        if (mr < 0.0f || (mr == 0.0f && mi < 0.0f)) m = -m, mr = -mr, mi = -mi;
-        float* q = w.rows + (o >> 1) * 16 + (o & 1);
-        q[0] = x1 ? px : py;
-        q[2] = y2 ? py : pz;
-        q[4] = t;
-        q[6] = -am;
-        q[8] = -lo;
-        q[10] = atan2f(mi, mr);
-        q[12] = m;
-        q[14] = 0.0f;
+        const float3 p = make_float3(fmaf(s1, s.e1[0], s2 * s.e2[0]), fmaf(s1, s.e1[1], s2 * s.e2[1]),
+                                     fmaf(s1, s.e1[2], s2 * s.e2[2]));
+        // m e^{i beta} with beta in [-pi/2, pi/2]: a negated moment negates m alone
+        float m = sqrtf(fmaf(m2.x, m2.x, m2.y * m2.y));
+        if (m2.x < 0.0f || (m2.x == 0.0f && m2.y < 0.0f)) m = -m, m2.x = -m2.x, m2.y = -m2.y;
+        model.node_record(b, rc, p, m, atan2f(m2.y, m2.x), w.rows + (o >> 1) * 16 + (o & 1));
     }
     __syncwarp();
     // -- node to node
     constexpr int G2 = node_groups<N>(), P2 = NN / 2, PER = (P2 + G2 - 1) / G2;
     float2* part = G2 > 1 ? w.y : w.x;
     static_assert(G2 * NN <= kMaxNN, "partial sums of the target nodes");
-    const float nx = s.e3[0], ny = s.e3[1], nz = s.e3[2];
 #pragma unroll 1
     for (int o2 = lane; o2 < NN * G2; o2 += 32) {
         const int gq = o2 / NN, o = o2 - gq * NN, a = o / N, c = o - a * N;
         const float q1 = 0.5f * N * C[a * N + 1] * b.q1, q2 = 0.5f * N * C[c * N + 1] * b.q2;
-        const float qx = x1 ? q1 : 0.0f, qy = (x1 ? 0.0f : q1) + (y2 ? q2 : 0.0f), qz = y2 ? 0.0f : q2;
-        // |d + q| = R + b as a sum of two floats
-        const float h = fmaf(qx, Dx, fmaf(qy, Dy, fmaf(qz, Dz, 0.5f * fmaf(q1, q1, q2 * q2))));
-        const float bq = path_diff(h, R, R2);
-        const float Rh = R + bq, Rl = bq - (Rh - R);
-        NodeRef n;
-        n.q1 = make_float2(-q1, -q1);
-        n.q2 = make_float2(-q2, -q2);
-        n.R2 = make_float2(Rh * Rh, Rh * Rh);
-        n.nR = make_float2(-Rh, -Rh);
-        n.nRh = make_float2(-0.5f * Rh, -0.5f * Rh);
-        const float cr = -__fdividef(Rl, Rh);
-        n.cr = make_float2(cr, cr);
-        float2 a1 = make_float2(0.f, 0.f), a2 = a1, b1 = a1, b2 = a1;
-        const float4* pr = reinterpret_cast<const float4*>(w.rows);
-        const int i1 = min(P2, (gq + 1) * PER);
-#pragma unroll 2
-        for (int i = gq * PER; i < i1; ++i)
-            node_pair2<KIND>(n, pr[4 * i], pr[4 * i + 1], pr[4 * i + 2], pr[4 * i + 3], k2, a1, a2, b1, b2);
-        float fr, fi;
-        if (KIND == RSI_STAGE_PISTON) {
-            fr = a1.x + a1.y;
-            fi = b1.x + b1.y;
-        } else {
-            // n . (Q - P) is the same for every source of a flat cluster
-            const float nd = fmaf(Dx + qx, nx, fmaf(Dy + qy, ny, (Dz + qz) * nz));
-            fr = nd * fmaf(-k, a2.x + a2.y, -(a1.x + a1.y));
-            fi = nd * fmaf(k, b2.x + b2.y, -(b1.x + b1.y));
-        }
-        // the moments carry e^{ik |d - p|} and the targets' phases e^{ik |d + q|}:
-        // one e^{ik |d|} too many
-        part[o2] = make_float2(fmaf(c0, fr, s0 * fi), fmaf(c0, fi, -s0 * fr));
+        const float2 f = model.node_field(s, b, rc, q1, q2, reinterpret_cast<const float4*>(w.rows), gq * PER,
+                                          min(P2, (gq + 1) * PER));
+        // the moments and the targets' phases each carry the factor of the centres: one too many
+        part[o2] = make_float2(fmaf(c0, f.x, s0 * f.y), fmaf(c0, f.y, -s0 * f.x));
     }
     __syncwarp();
     if (G2 > 1) {
@@ -633,61 +549,142 @@ __device__ __forceinline__ void add_comp(float4& acc, float ar, float ai) {
     acc.w = __fadd_rn(acc.w, e);
 }
 
-// the direct sum of a staged tile at T targets of this thread (quarters apart)
-template <int KIND, int NORM, int T>
-__device__ __forceinline__ void direct_tile(const Sum& g, const float* hdr, const float4* rec, const int* slot,
-                                            float4* acc) {
-    const float k = g.kh, far_min = 2.0f * hdr[6];
-    bool far_lane = true;
-    rsi_fp32::TgtRef2 r2[T];
-    float tau[T];
-    float2 a1[T], a2[T], b1[T], b2[T];
-#pragma unroll
-    for (int q = 0; q < T; ++q) {
-        const int j = slot[q * kThreads];
+// What a sum's pair terms are: the interface that warp_item and run_block need,
+// for the piston and Rayleigh-Sommerfeld stages.  (raytrace.cu has its own.)
+template <int KIND, int NORM>
+struct StageModel {
+    static constexpr bool kPolar = KIND == RSI_STAGE_RSI;  // source amplitudes m e^{i beta}, or real
+    static constexpr int kDirectCost = 134;  // instructions per warp of a tile's source onto 256 targets, direct
+    using Ref = rsi_fp32::TgtRef;
+    const Sum& g;
+
+    __device__ __forceinline__ int choose(const Node& s, const Box& b) const { return choose_nodes(s, b, g.kh); }
+    __device__ __forceinline__ static float cost(float ns, float nt, int N) { return pair_cost(ns, nt, N, 36.f, 85.f, 75.f); }
+    __device__ __forceinline__ Ref reference(const float* t, const float* c) const {
+        return rsi_fp32::target_reference(t[0], t[1], t[2], t[3], t[4], t[5], c, g.kh, g.kl, g.tp);
+    }
+    __device__ __forceinline__ Ref broadcast(const Ref& r, int lane) const {
+        Ref o;
+        o.Dx = __shfl_sync(0xffffffffu, r.Dx, lane);
+        o.Dy = __shfl_sync(0xffffffffu, r.Dy, lane);
+        o.Dz = __shfl_sync(0xffffffffu, r.Dz, lane);
+        o.R = __shfl_sync(0xffffffffu, r.R, lane);
+        o.tau = 0.318309886f * __shfl_sync(0xffffffffu, r.tau, lane);  // half turns
+        o.R2 = o.R * o.R;
+        return o;
+    }
+    // k |d - p| of two sources in half turns, less whole turns
+    __device__ __forceinline__ float2 source_phase(const Ref& r, float2 px, float2 py, float2 pzn, float2 pw) const {
+        const float2 magic = dup(12582912.0f), nmagic = dup(-12582912.0f);  // 1.5 2^23: rounds to an integer
+        const float2 th = __ffma2_rn(dup(-r.Dx), px, __ffma2_rn(dup(-r.Dy), py, __ffma2_rn(dup(r.Dz), pzn, pw)));
+        const float2 r2 = __ffma2_rn(th, dup(2.0f), dup(r.R2));
+        const float2 ir = make_float2(rsqrt_approx(r2.x), rsqrt_approx(r2.y));
+        const float2 r0 = __fmul2_rn(r2, ir);
+        const float2 am = __fadd2_rn(r0, dup(-r.R));
+        const float2 a = __ffma2_rn(__ffma2_rn(am, __ffma2_rn(r0, dup(-0.5f), dup(-0.5f * r.R)), th), ir, am);
+        const float2 ph = __fmul2_rn(dup(g.kph), a);
+        const float2 pl = __ffma2_rn(dup(g.kpl), a, __ffma2_rn(dup(g.kph), a, __fmul2_rn(dup(-g.kph), a)));
+        const float2 x = __ffma2_rn(__fadd2_rn(__ffma2_rn(ph, dup(0.5f), magic), nmagic), dup(-2.0f), ph);
+        return __fadd2_rn(x, __fadd2_rn(pl, dup(r.tau)));
+    }
+    // for the targets' phases: the block's centre from the cluster's, exactly (one lane)
+    __device__ __forceinline__ void prepare_targets(WarpArea& w, const Box& b, const Box& b0) const {
+        if (threadIdx.x & 31) return;
+        const Node& s = w.node;
+        float dh[3], dl[3], sh[3], sl[3];
+        for (int q = 0; q < 3; ++q) {
+            df_diff(b0.c[2 * q], b0.c[2 * q + 1], s.c[2 * q], s.c[2 * q + 1], dh[q], dl[q]);
+            df_sqr(dh[q], dl[q], sh[q], sl[q]);
+        }
+        df_add_pos(sh[0], sl[0], sh[1], sl[1], sh[0], sl[0]);
+        df_add_pos(sh[0], sl[0], sh[2], sl[2], w.S0h, w.S0l);
+        w.D1h = b.ax1 == 0 ? dh[0] : dh[1], w.D1l = b.ax1 == 0 ? dl[0] : dl[1];
+        w.D2h = b.ax2 == 1 ? dh[1] : dh[2], w.D2l = b.ax2 == 1 ? dl[1] : dl[2];
+    }
+    __device__ __forceinline__ void centre_phase(const WarpArea& w, const Box& b, const Box& b0, const Ref&, float& c,
+                                                 float& s) const {
+        TargetPos t;
+        df_diff(b.c[2 * b.ax1], b.c[2 * b.ax1 + 1], b0.c[2 * b.ax1], b0.c[2 * b.ax1 + 1], t.q1h, t.q1l);
+        df_diff(b.c[2 * b.ax2], b.c[2 * b.ax2 + 1], b0.c[2 * b.ax2], b0.c[2 * b.ax2 + 1], t.q2h, t.q2l);
+        float a1, e1, a2, e2;
+        df_sqr(t.q1h, t.q1l, a1, e1);
+        df_sqr(t.q2h, t.q2l, a2, e2);
+        df_add_pos(a1, e1, a2, e2, t.sh, t.sl);
+        target_phase(w, t, g.kph, g.kpl, c, s);
+    }
+    __device__ __forceinline__ void target(const WarpArea& w, const TargetPos& t, int, float& c, float& s) const {
+        target_phase(w, t, g.kph, g.kpl, c, s);
+    }
+    // the record of a source node at p (node_pair2), pair-interleaved
+    __device__ __forceinline__ void node_record(const Box& b, const Ref& r, const float3& p, float m, float beta,
+                                                float* q) const {
+        const float t = fmaf(-r.Dx, p.x, fmaf(-r.Dy, p.y, fmaf(-r.Dz, p.z, 0.5f * fmaf(p.x, p.x, fmaf(p.y, p.y, p.z * p.z)))));
+        // a = |d - p| - |d| for this t as a sum of two floats: r0 - R is exact, the Newton correction small
+        const float r2 = fmaf(2.0f, t, r.R2), ir = rsqrt_approx(r2), r0 = r2 * ir, am = r0 - r.R;
+        q[0] = b.ax1 == 0 ? p.x : p.y;
+        q[2] = b.ax2 == 1 ? p.y : p.z;
+        q[4] = t;
+        q[6] = -am;
+        q[8] = -(fmaf(am, -0.5f * (r0 + r.R), t) * ir);
+        q[10] = beta;
+        q[12] = m;
+        q[14] = 0.0f;
+    }
+    // the field of source nodes 2 i0 .. 2 i1 - 1 at the target node (q1, q2) of the box
+    __device__ __forceinline__ float2 node_field(const Node& s, const Box& b, const Ref& r, float q1, float q2,
+                                                 const float4* pr, int i0, int i1) const {
+        const bool x1 = b.ax1 == 0, y2 = b.ax2 == 1;
+        const float qx = x1 ? q1 : 0.0f, qy = (x1 ? 0.0f : q1) + (y2 ? q2 : 0.0f), qz = y2 ? 0.0f : q2;
+        // |d + q| = R + b as a sum of two floats
+        const float h = fmaf(qx, r.Dx, fmaf(qy, r.Dy, fmaf(qz, r.Dz, 0.5f * fmaf(q1, q1, q2 * q2))));
+        const float bq = path_diff(h, r.R, r.R2);
+        const float Rh = r.R + bq, Rl = bq - (Rh - r.R);
+        NodeRef n;
+        n.q1 = dup(-q1);
+        n.q2 = dup(-q2);
+        n.R2 = dup(Rh * Rh);
+        n.nR = dup(-Rh);
+        n.nRh = dup(-0.5f * Rh);
+        n.cr = dup(-__fdividef(Rl, Rh));
+        const float2 k2 = dup(g.kh);
+        float2 a1 = make_float2(0.f, 0.f), a2 = a1, b1 = a1, b2 = a1;
+#pragma unroll 2
+        for (int i = i0; i < i1; ++i)
+            node_pair2<KIND>(n, pr[4 * i], pr[4 * i + 1], pr[4 * i + 2], pr[4 * i + 3], k2, a1, a2, b1, b2);
+        if (KIND == RSI_STAGE_PISTON) return make_float2(a1.x + a1.y, b1.x + b1.y);
+        // n . (Q - P) is the same for every source of a flat cluster
+        const float nd = fmaf(r.Dx + qx, s.e3[0], fmaf(r.Dy + qy, s.e3[1], (r.Dz + qz) * s.e3[2]));
+        return make_float2(nd * fmaf(-g.kh, a2.x + a2.y, -(a1.x + a1.y)), nd * fmaf(g.kh, b2.x + b2.y, -(b1.x + b1.y)));
+    }
+    // the direct sum of a staged tile at target j
+    __device__ __forceinline__ float2 direct(const float* hdr, const float4* rec, int64_t j) const {
         const rsi_fp32::TgtRef ref = rsi_fp32::target_reference(
             __ldg(g.tgt.xh + j), __ldg(g.tgt.xl + j), __ldg(g.tgt.yh + j), __ldg(g.tgt.yl + j), __ldg(g.tgt.zh + j),
             __ldg(g.tgt.zl + j), hdr, g.kh, g.kl, g.tp);
-        far_lane = far_lane && ref.R > far_min && ref.R > 0.0f;
-        r2[q] = rsi_fp32::packed_reference(ref);
-        tau[q] = ref.tau;
-        a1[q] = a2[q] = b1[q] = b2[q] = make_float2(0.f, 0.f);
+        const bool far_lane = ref.R > 2.0f * hdr[6] && ref.R > 0.0f;
+        const rsi_fp32::TgtRef2 r2[1] = {rsi_fp32::packed_reference(ref)};
+        float2 a1[1], a2[1], b1[1], b2[1];
+        a1[0] = a2[0] = b1[0] = b2[0] = make_float2(0.f, 0.f);
+        const float k = g.kh;
+        if (__all_sync(0xffffffffu, far_lane))
+            rsi_fp32::packed_tile<KIND, NORM, 1, false>(rec, g.S, r2, dup(k), a1, a2, b1, b2);
+        else
+            rsi_fp32::packed_tile<KIND, NORM, 1, true>(rec, g.S, r2, dup(k), a1, a2, b1, b2);
+        if (KIND == RSI_STAGE_PISTON) return make_float2(a1[0].x + a1[0].y, b1[0].x + b1[0].y);
+        const float sr = fmaf(-k, a2[0].x + a2[0].y, -(a1[0].x + a1[0].y));
+        const float si = fmaf(k, b2[0].x + b2[0].y, -(b1[0].x + b1[0].y));
+        float st, ct;
+        __sincosf(ref.tau, &st, &ct);
+        return make_float2(fmaf(ct, sr, -st * si), fmaf(st, sr, ct * si));
     }
-    const float2 k2 = make_float2(k, k);
-    if (__all_sync(0xffffffffu, far_lane))
-        rsi_fp32::packed_tile<KIND, NORM, T, false>(rec, g.S, r2, k2, a1, a2, b1, b2);
-    else
-        rsi_fp32::packed_tile<KIND, NORM, T, true>(rec, g.S, r2, k2, a1, a2, b1, b2);
-#pragma unroll
-    for (int q = 0; q < T; ++q) {
-        float ar, ai;
-        if (KIND == RSI_STAGE_PISTON) {
-            ar = a1[q].x + a1[q].y;
-            ai = b1[q].x + b1[q].y;
-        } else {
-            const float sr = fmaf(-k, a2[q].x + a2[q].y, -(a1[q].x + a1[q].y));
-            const float si = fmaf(k, b2[q].x + b2[q].y, -(b1[q].x + b1[q].y));
-            float st, ct;
-            __sincosf(tau[q], &st, &ct);
-            ar = fmaf(ct, sr, -st * si);
-            ai = fmaf(st, sr, ct * si);
-        }
-        float4 a = acc[q * kThreads];
-        add_comp(a, ar, ai);
-        acc[q * kThreads] = a;
-    }
-}
+};
 
-__device__ __forceinline__ void init_shared(Shared& sh, uint64_t* bars) {
+__device__ __forceinline__ void init_shared(Shared& sh) {
     for (int e = threadIdx.x; e < kTabFloats; e += kThreads) {
         const int n = e < 36 ? 6 : e < 100 ? 8 : e < 200 ? 10 : 12;
         const int o = e - tab_off(n), a = o / n, kk = o - a * n;
         const float v = (kk ? 2.0f : 1.0f) / float(n) * cospif(float((2 * a + 1) * kk) / float(2 * n));
         sh.tab[e] = kk & 2 ? -v : v;
-    }
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < 2; ++s) mbar_init(smem_u32(&bars[s]), 1);
-        fence_mbar_init();
     }
     __syncthreads();
 }
@@ -715,15 +712,13 @@ __device__ __forceinline__ int block_scan(int n, Shared& sh, int& total) {
 }
 
 // One CTA: targets t0 .. t0 + 256 TPT - 1 of the block order against the root
-// clusters (16 tiles) r_first, r_first + r_step, ...; acc and uv hold one
-// entry per target.  Returns false (after recording RSI_DEV_TIMEOUT) if a
-// bounded wait expired.  `uses` counts the tile-buffer fills of this CTA.
-template <int KIND, int NORM, int TPT>
-__device__ __forceinline__ bool run_block(const Sum& g, int64_t t0, int r_first, int r_step, int L, int h,
-                                          double2* out, Shared& sh, float4* acc, int* slot, uint64_t* bars,
-                                          uint32_t& uses) {
+// clusters (16 tiles) r_first, r_first + r_step, ...; acc and slot hold one
+// entry per target.  left[tile]: the quarters of the block that the tile's
+// direct sum is left for (leftover_block); *any is raised where there are some.
+template <class M, int TPT>
+__device__ __forceinline__ void run_block(const M& model, const Sum& g, int64_t t0, int r_first, int r_step, int L, int h,
+                                          double2* out, uint8_t* left, int* any, Shared& sh, float4* acc, int* slot) {
     const int tid = threadIdx.x, warp = tid >> 5;
-    const float k = g.kh;
     if (tid < int(5 * sizeof(Box) / 4))
         reinterpret_cast<float*>(sh.box)[tid] = __ldg(reinterpret_cast<const float*>(g.boxes + 5 * (t0 / (TPT * kThreads))) + tid);
     __syncthreads();
@@ -742,7 +737,7 @@ __device__ __forceinline__ bool run_block(const Sum& g, int64_t t0, int r_first,
         int lev = -1, n = 0, quarters[4] = {0, 0, 0, 0}, emit = 0, mask = 0;
         if (root < n_roots && tile < g.n_tiles) {
             for (int l = g.top; l >= 0 && !n; --l) {
-                n = choose_nodes(g.nodes[l][tile >> (2 * l)], sh.box[0], k);
+                n = model.choose(g.nodes[l][tile >> (2 * l)], sh.box[0]);
                 lev = l;
             }
             if (n) {
@@ -750,7 +745,7 @@ __device__ __forceinline__ bool run_block(const Sum& g, int64_t t0, int r_first,
             } else {
                 lev = 0;
                 for (int q = 0; q < TPT && TPT > 1; ++q) {
-                    quarters[q] = choose_nodes(g.nodes[0][tile], sh.box[1 + q], k);
+                    quarters[q] = model.choose(g.nodes[0][tile], sh.box[1 + q]);
                     if (quarters[q])
                         ++emit;
                     else
@@ -781,9 +776,8 @@ __device__ __forceinline__ bool run_block(const Sum& g, int64_t t0, int r_first,
             }
             at += total;
         }
-        int n_direct;
-        const int dpos = block_scan(mask != 0, sh, n_direct);
-        if (mask) sh.direct[dpos] = (tile << 4) | mask;
+        if (root < n_roots && tile < g.n_tiles) left[tile] = uint8_t(mask);
+        if (mask) *any = 1;
         const int n_items = at;
         __syncthreads();
 
@@ -800,10 +794,10 @@ __device__ __forceinline__ bool run_block(const Sum& g, int64_t t0, int r_first,
                 const Box& b = sh.box[(item >> 4) & 7];
                 const int nt = min(1 << (2 * lev_i), g.n_tiles - t_i);
                 switch (N) {
-                    case 6: warp_item<KIND, 6>(g, b, sh.box[0], t_i, nt, w, sh.tab); break;
-                    case 8: warp_item<KIND, 8>(g, b, sh.box[0], t_i, nt, w, sh.tab); break;
-                    case 10: warp_item<KIND, 10>(g, b, sh.box[0], t_i, nt, w, sh.tab); break;
-                    default: warp_item<KIND, 12>(g, b, sh.box[0], t_i, nt, w, sh.tab); break;
+                    case 6: warp_item<M, 6>(model, g, b, sh.box[0], t_i, nt, w, sh.tab); break;
+                    case 8: warp_item<M, 8>(model, g, b, sh.box[0], t_i, nt, w, sh.tab); break;
+                    case 10: warp_item<M, 10>(model, g, b, sh.box[0], t_i, nt, w, sh.tab); break;
+                    default: warp_item<M, 12>(model, g, b, sh.box[0], t_i, nt, w, sh.tab); break;
                 }
             }
             __syncthreads();
@@ -847,7 +841,7 @@ __device__ __forceinline__ bool run_block(const Sum& g, int64_t t0, int r_first,
                     for (int q = 0; q < T; ++q) {
                         if (bx && bx - 1 != q0 + q) continue;
                         float st, ct;
-                        target_phase(wi, tp[q], g.kph, g.kpl, ct, st);
+                        model.target(wi, tp[q], slot[(q0 + q) * kThreads + tid], ct, st);
                         add_comp(a[q], fmaf(ct, f[q].x, -st * f[q].y), fmaf(st, f[q].x, ct * f[q].y));
                     }
                 }
@@ -857,49 +851,6 @@ __device__ __forceinline__ bool run_block(const Sum& g, int64_t t0, int r_first,
             __syncthreads();
         }
 
-        // -- direct sums of the tiles and quarters left over; the tile buffers take the warps' areas
-        uint8_t* buf = reinterpret_cast<uint8_t*>(sh.w);
-        const uint32_t stride = (g.tile_bytes + 127u) & ~127u;
-        auto fetch = [&](int i) {
-            if (tid == 0 && i < n_direct) {
-                const uint32_t u = (uses + i) & 1u, bar = smem_u32(&bars[u]);
-                mbar_expect_tx(bar, g.tile_bytes);
-                bulk_g2s(smem_u32(buf + u * stride), g.tiles + size_t(sh.direct[i] >> 4) * g.tile_bytes, g.tile_bytes,
-                         bar);
-            }
-        };
-        if (n_direct && tid == 0) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        fetch(0);
-        fetch(1);
-        for (int i = 0; i < n_direct; ++i) {
-            const uint32_t u = uses + i;
-            const bool ok = mbar_wait_bounded(smem_u32(&bars[u & 1u]), (u >> 1) & 1u);
-            if (__syncthreads_or(!ok)) {
-                if (tid == 0) {
-                    atomicExch(g.status, RSI_DEV_TIMEOUT);
-                    for (int e = i; e < n_direct && e < i + 2; ++e)
-                        mbar_wait_bounded(smem_u32(&bars[(uses + e) & 1u]), ((uses + e) >> 1) & 1u);
-                }
-                return false;
-            }
-            const uint8_t* tl = buf + (u & 1u) * stride;
-            const float* hdr = reinterpret_cast<const float*>(tl);
-            const float4* rec = reinterpret_cast<const float4*>(tl + RSI_TILE_HDR_BYTES);
-            const int msk = sh.direct[i] & 15;
-#pragma unroll 1
-            for (int q = 0; q < TPT; q += 2) {
-                const int m2 = (msk >> q) & 3;
-                if (TPT > 1 && m2 == 3)
-                    direct_tile<KIND, NORM, 2>(g, hdr, rec, slot + q * kThreads + tid, acc + q * kThreads + tid);
-                else if (m2)
-                    direct_tile<KIND, NORM, 1>(g, hdr, rec, slot + (q + (m2 >> 1)) * kThreads + tid,
-                                               acc + (q + (m2 >> 1)) * kThreads + tid);
-            }
-            __syncthreads();  // every thread is done with this buffer
-            fetch(i + 2);
-        }
-        uses += uint32_t(n_direct);
-        __syncthreads();  // before the lists and the warps' areas are written again
     }
 #pragma unroll
     for (int q = 0; q < TPT; ++q) {
@@ -907,10 +858,98 @@ __device__ __forceinline__ bool run_block(const Sum& g, int64_t t0, int r_first,
         if (t >= g.n_tgt) continue;
         const float4 a = acc[q * kThreads + tid];
         const double re = double(a.x) + double(a.y), im = double(a.z) + double(a.w);
-        if (!isfinite(re) || !isfinite(im)) atomicExch(g.status, RSI_DEV_NONFINITE);
         out[slot[q * kThreads + tid]] = make_double2(re, im);
     }
-    return true;
+}
+
+// ---------------------------------------------------------------------------
+// What the clusters leave: a CTA takes the 256 targets of one quarter (t0 in
+// the block order) and the tiles seg, seg + segs, ... whose `left` mask has the
+// quarter's bit, in the direct kernel's manner (bulk copies kPipe deep, one
+// target a thread, 4 CTAs per SM).  A kernel of its own: the leftovers of the
+// blocks at the sources are most of the work where there are any, and spread
+// over the whole GPU like this they take the direct kernel's time per pair
+// (inside the clustered kernel the ray-tracing image took 27.6 ms, 16 blocks
+// next to the interface holding up the rest).
+// ---------------------------------------------------------------------------
+constexpr int kPipe = RSI_PIPE_STAGES;
+__host__ __device__ constexpr size_t leftover_smem(size_t tile_bytes) {
+    return kPipe * tile_bytes + kPipe * sizeof(uint64_t);
+}
+template <class M, int TPT>
+__device__ __forceinline__ void leftover_block(const M& model, const Sum& g, int64_t block, int quarter, int seg, int segs,
+                                               int L, int h, const uint8_t* __restrict__ left, double2* out,
+                                               uint8_t* smem) {
+    __shared__ int list[kRound];
+    __shared__ int warp_sum[kWarps];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kPipe * g.tile_bytes);
+    if (tid == 0) {
+        for (int s = 0; s < kPipe; ++s) mbar_init(smem_u32(&bars[s]), 1);
+        fence_mbar_init();
+    }
+    __syncthreads();
+    const int64_t t = block * TPT * kThreads + block_pos<TPT>(quarter * kThreads + tid, h);
+    const int64_t j = strip_slot(t < g.n_tgt ? t : g.n_tgt - 1, g.n_tgt, L, h);
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    uint32_t uses = 0;
+    for (int r0 = 0; seg + r0 * segs < g.n_tiles; r0 += kRound) {
+        const int tile = seg + (r0 + tid) * segs;
+        const bool mine = tile < g.n_tiles && ((left[tile] >> quarter) & 1);
+        const unsigned vote = __ballot_sync(0xffffffffu, mine);
+        if (lane == 0) warp_sum[wid] = __popc(vote);
+        __syncthreads();
+        int at = 0, n = 0;
+        for (int q = 0; q < kWarps; ++q) {
+            at += q < wid ? warp_sum[q] : 0;
+            n += warp_sum[q];
+        }
+        if (mine) list[at + __popc(vote & ((1u << lane) - 1u))] = tile;
+        __syncthreads();
+        auto fetch = [&](int i) {
+            if (tid == 0 && i < n) {
+                const uint32_t u = (uses + i) % kPipe, bar = smem_u32(&bars[u]);
+                mbar_expect_tx(bar, g.tile_bytes);
+                bulk_g2s(smem_u32(smem + u * g.tile_bytes), g.tiles + size_t(list[i]) * g.tile_bytes, g.tile_bytes, bar);
+            }
+        };
+        for (int s = 0; s < kPipe; ++s) fetch(s);
+        for (int i = 0; i < n; ++i) {
+            const uint32_t u = uses + i;
+            const bool ok = mbar_wait_bounded(smem_u32(&bars[u % kPipe]), (u / kPipe) & 1u);
+            if (__syncthreads_or(!ok)) {
+                if (tid == 0) {
+                    atomicExch(g.status, RSI_DEV_TIMEOUT);
+                    for (int e = i; e < n && e < i + kPipe; ++e)
+                        mbar_wait_bounded(smem_u32(&bars[(uses + e) % kPipe]), ((uses + e) / kPipe) & 1u);
+                }
+                return;
+            }
+            const uint8_t* tl = smem + (u % kPipe) * g.tile_bytes;
+            const float2 f = model.direct(reinterpret_cast<const float*>(tl),
+                                          reinterpret_cast<const float4*>(tl + RSI_TILE_HDR_BYTES), j);
+            add_comp(acc, f.x, f.y);
+            __syncthreads();  // every thread is done with this buffer
+            fetch(i + kPipe);
+        }
+        uses += uint32_t(n);
+    }
+    if (t < g.n_tgt) out[j] = make_double2(double(acc.x) + double(acc.y), double(acc.z) + double(acc.w));
+}
+
+// The partial sums of `splits` clustered CTAs and, where the block has
+// leftovers, of `segs` leftover CTAs (after them) at the t-th target of the
+// block order (Neumaier, in order).
+template <int TPT>
+__device__ __forceinline__ void sum_block_order(const double2* __restrict__ part, int splits, int segs,
+                                                const int* __restrict__ any, int64_t t, int64_t n, int L, int h,
+                                                double2* __restrict__ out, int* status) {
+    if (t >= (n + TPT * kThreads - 1) / (TPT * kThreads) * (TPT * kThreads)) return;
+    const int64_t block = t / (TPT * kThreads);
+    const int64_t u = block * TPT * kThreads + block_pos<TPT>(int(t - block * TPT * kThreads), h);
+    if (u >= n) return;
+    const int64_t j = strip_slot(u, n, L, h);
+    sum_partials(part + j, splits + (any[block] ? segs : 0), n, out + j, status);
 }
 
 // ---------------------------------------------------------------------------
@@ -1014,21 +1053,27 @@ __device__ __forceinline__ void make_node(int kind, int normals, const PointsVie
 // CTA measures it for itself, which costs less than a launch that does it once.
 __device__ __forceinline__ int source_mode(int kind, const PointsView& src, int64_t n, float* red) {
     if (kind != RSI_STAGE_PISTON || n < 4096) return 0;
+    const int warp = threadIdx.x >> 5, run = warp >> 1, mode = warp & 1;  // 8 warps: a run in one of the orders each
+    // places without a common factor with the cells' sizes
+    const int64_t i0 = n / 1024 * ((317 + 631 * run) % 1021) / 256 * 256;
+    float e[6] = {INFINITY, INFINITY, INFINITY, INFINITY, INFINITY, INFINITY};
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const int64_t j = rsi_fp32::source_slot(i0 + q * 32 + (threadIdx.x & 31), n, mode);
+        const float x = src.xh[j], y = src.yh[j], z = src.zh[j];
+        e[0] = fminf(e[0], x), e[1] = fminf(e[1], y), e[2] = fminf(e[2], z);
+        e[3] = fminf(e[3], -x), e[4] = fminf(e[4], -y), e[5] = fminf(e[5], -z);
+    }
+#pragma unroll
+    for (int q = 0; q < 6; ++q)
+#pragma unroll
+        for (int o = 16; o; o >>= 1) e[q] = fminf(e[q], __shfl_xor_sync(0xffffffffu, e[q], o));
+    const float x = -e[3] - e[0], y = -e[4] - e[1], z = -e[5] - e[2];
+    if ((threadIdx.x & 31) == 0) red[warp] = fmaf(x, x, fmaf(y, y, z * z));
+    __syncthreads();
     float size[2] = {0.0f, 0.0f};
-    for (int run = 0; run < 4; ++run)
-        for (int mode = 0; mode < 2; ++mode) {
-            // places without a common factor with the cells' sizes
-            const int64_t i0 = n / 1024 * ((317 + 631 * run) % 1021) / 256 * 256;
-            float e[6] = {INFINITY, INFINITY, INFINITY, INFINITY, INFINITY, INFINITY};
-            if (threadIdx.x < 256) {
-                const int64_t j = rsi_fp32::source_slot(i0 + threadIdx.x, n, mode);
-                const float x = src.xh[j], y = src.yh[j], z = src.zh[j];
-                e[0] = x, e[1] = y, e[2] = z, e[3] = -x, e[4] = -y, e[5] = -z;
-            }
-            rsi_fp32::block_min6(e, red);
-            const float x = -e[3] - e[0], y = -e[4] - e[1], z = -e[5] - e[2];
-            size[mode] += fmaf(x, x, fmaf(y, y, z * z));
-        }
+    for (int q = 0; q < 8; ++q) size[q & 1] += red[q];
+    __syncthreads();
     return size[1] < 0.9f * size[0] ? 1 : 0;
 }
 
@@ -1115,10 +1160,12 @@ __device__ __forceinline__ void find_rows(const TgtView& tgt, int64_t n, int per
 }
 
 // Adds one CTA's share of the cost estimate: a block of targets against up to
-// 256 tiles, one a thread.
-template <int TPT>
-__device__ __forceinline__ void estimate(const Node* nodes, int n_tiles, int S, int top, const Box* box, float k,
-                                         unsigned cta, StageGate* gate) {
+// 256 tiles, one a thread.  `weight`: of the clustered kernel's instructions
+// beside the direct sum's.
+template <class M, int TPT>
+__device__ __forceinline__ void estimate(const M& model, const Node* nodes, int n_tiles, int S, int top,
+                                         const Box* box, float weight, unsigned cta,
+                                         StageGate* gate) {
     const int samples = min(n_tiles, kThreads);
     const Node* lev[kLevels] = {nodes, nodes + n_tiles, nodes + n_tiles + (n_tiles + 3) / 4};
     float cost = 0.0f;
@@ -1127,13 +1174,13 @@ __device__ __forceinline__ void estimate(const Node* nodes, int n_tiles, int S, 
             int((int64_t(threadIdx.x) * n_tiles / samples + int64_t(cta) * n_tiles / (16 * samples)) % n_tiles);
         int n = 0, l = top;
         for (; l >= 0; --l)
-            if ((n = choose_nodes(lev[l][tile >> (2 * l)], box[0], k)) != 0) break;
+            if ((n = model.choose(lev[l][tile >> (2 * l)], box[0])) != 0) break;
         if (n) {
             const float units = float(1 << (2 * l));
-            cost = pair_cost(float(S) * units, float(TPT * kThreads), n) / (units * TPT);
+            cost = weight * M::cost(float(S) * units, float(TPT * kThreads), n) / (units * TPT);
         } else {
-            const int m = TPT > 1 ? choose_nodes(lev[0][tile], box[1 + threadIdx.x % TPT], k) : 0;
-            cost = m ? pair_cost(float(S), float(kThreads), m) : 134.4f * S;
+            const int m = TPT > 1 ? model.choose(lev[0][tile], box[1 + threadIdx.x % TPT]) : 0;
+            cost = m ? weight * M::cost(float(S), float(kThreads), m) : float(M::kDirectCost) * S;
         }
     }
     __shared__ unsigned sum;

@@ -7,10 +7,12 @@ of the direct sum's terms, about 1e-6; incoherent over the clusters, the
 relative L2 error of a field stays below 5e-6 plus what the direct kernel has."""
 import math
 
+import numpy as np
 import pytest
 import torch
 
-from paper_2408_06765_gb300 import build, rsi
+import oracle
+from paper_2408_06765_gb300 import build, rsi, workloads
 
 pytestmark = pytest.mark.gpu
 TOL = 5e-6
@@ -107,3 +109,27 @@ def test_stages_without_clusters_take_the_direct_kernel(case):
     a, b = (rsi.propagate_stage(rsi.stage_struct(rsi.STAGE_RSI, "fp32c", k, variant=v), src, sigma, tgt) for v in (0, 3))
     rsi.sync_status()
     assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("case", ["steep", "ragged", "into the slower medium", "near the interface"])
+def test_raytrace_matches_direct_and_oracle(case):
+    """The clustered ray-tracing sum against the direct one (a given tile) and the FP64 oracle at pixels over the image, by the same
+    tolerance: edges of tiles and blocks, rows off the block's strips, rays
+    close to the plane (left to the direct sum) and up to 75 degrees."""
+    n, nx, nz = {"steep": (16384, 256, 96), "ragged": (9001, 257, 171)}.get(case, (20011, 131, 130))
+    cfg = workloads.f2_ray_tracing(n_piston=n, nx=nx, nz=nz)
+    g, zi = cfg["grid"], float(cfg["interfaces"][0]["centre"][2])
+    if case == "steep":
+        g.update({"x0": -0.03, "x1": 0.03})
+    elif case == "into the slower medium":
+        cfg["media"] = cfg["media"][::-1]
+    elif case == "near the interface":
+        g.update({"z0": zi + 1e-5, "z1": zi + 0.02})
+    clustered, direct = rsi.run_raytrace(cfg), rsi.run_raytrace(cfg, tile=128 if n == 9001 else 256)
+    rsi.sync_status()
+    assert not torch.equal(clustered, direct)
+    assert rel(clustered, direct) <= TOL
+    px = np.linspace(0, nx * nz - 1, 64).astype(np.int64)
+    want = torch.from_numpy(oracle.raytrace_image(cfg, pixels=px))
+    got, ref = (v.reshape(-1).cpu()[torch.from_numpy(px)] for v in (clustered, direct))
+    assert rel(got, want) <= rel(ref, want) + TOL
