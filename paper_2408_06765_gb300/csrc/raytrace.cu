@@ -959,7 +959,7 @@ extern "C" int rsi_raytrace_field(const rsi_raytrace* rt, const void* src_points
         c.gate = reinterpret_cast<StageGate*>(extra + p.c.extra_bytes - 256);
         c.field = field;
         a.gate = c.gate;
-        a.gate_ratio = float(RayModel::kDirectCost) / 134.4f;
+        a.gate_ratio = p.c.gain * (float(RayModel::kDirectCost) / 134.4f);
         c.weight = kClusterWeight / p.c.fill;
         c.a = a;
         c.a.splits = p.c.splits;

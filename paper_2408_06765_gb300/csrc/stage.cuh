@@ -117,6 +117,7 @@ struct ClusterPlan {
     int nf, n_tiles, S, splits, top;
     int segs;    // CTAs per quarter block for the leftovers
     float fill;  // share of the GPU's CTA slots that the launch fills
+    float gain;  // share of the direct sum's time that the clusters' arithmetic may take
     size_t tile_bytes, tiles_bytes, extra_bytes, partial_bytes;  // tiles and partial sums: of one frequency
     size_t boxes_at, left_at, any_at;  // within extra
     size_t total() const { return size_t(nf) * (tiles_bytes + partial_bytes) + extra_bytes; }

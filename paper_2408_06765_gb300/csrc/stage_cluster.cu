@@ -175,16 +175,18 @@ size_t nodes_bytes(int n_tiles) {
 
 }  // namespace
 
-// Clusters pay where the sum is long: preparation and estimate take about 15 us
-// more than the direct kernel's preparation, and 4e8 pairs take that kernel
-// 0.3 ms.  A piston's clusters are small beside the distance and nearly always
+// Clusters pay where the sum is long: preparation, estimate and the launches take
+// about 40 us more than the direct kernel's, and 6e8 pairs take that kernel
+// 0.45 ms.  A piston's clusters are small beside the distance and nearly always
 // taken; an interface's may not be, so its sums have to be longer, and those of
-// several frequencies, whose direct sum is shared, twice as long; a ray costs the
-// direct kernel 6 times a stage's pair.  Per-point normals turn within a
+// several frequencies, whose direct sum is shared, three times as long (9e8 and
+// 7.8e8 pairs at three frequencies: 2.25 and 1.5 ms either way, less the 40 us);
+// a ray costs the direct kernel 7 times a stage's pair (16384 x 256 x 128:
+// 2.32 -> 1.81 ms, 9001 x 101 x 77: 0.55 -> 1.29 ms).  Per-point normals turn within a
 // tile on every curved surface, where the direct sum would be taken anyway.
 bool cluster_plan(int kind, int normals, int nf, int64_t n_src, int64_t n_tgt, int S, int splits, int max_auto_splits,
                   ClusterPlan& p) {
-    const double least = kind == RSI_TIMING_RAYTRACE ? 3e8 : (kind == RSI_STAGE_PISTON ? 4e8 : 1e9) * (nf > 1 ? 2.0 : 1.0);
+    const double least = kind == RSI_TIMING_RAYTRACE ? 3e8 : (kind == RSI_STAGE_PISTON ? 6e8 : 1e9) * (nf > 1 ? 3.0 : 1.0);
     if (n_src < 8192 || n_tgt < 4096 || double(n_src) * double(n_tgt) < least) return false;
     if (kind == RSI_STAGE_RSI && base_normals(normals) != RSI_NORMALS_Z) return false;
     const int n_tiles = int((n_src + S - 1) / S);
@@ -222,6 +224,11 @@ bool cluster_plan(int kind, int normals, int nf, int64_t n_src, int64_t n_tgt, i
     p.splits = int((roots + rps - 1) / rps);
     p.top = top(rps);
     p.fill = float(std::min(1.0, double(blocks * p.splits * nf) / double(slots)));
+    // what the 60 us of launches and CTAs' set-up, at 9.2e11 instructions per warp
+    // and second, leave of the direct sum's time for the clusters' arithmetic
+    // (134.4 instructions per source and 256 targets)
+    const double direct = (kind == RSI_TIMING_RAYTRACE ? 976.0 : 134.4) * double(n_src) * double(blocks * kTpt) * nf;
+    p.gain = float(std::max(0.0, 1.0 - 5.5e7 / direct));
     p.tile_bytes = RSI_TILE_HDR_BYTES + size_t(S) * fp32_record_bytes(kind, base_normals(normals));
     p.tiles_bytes = align256(size_t(n_tiles) * p.tile_bytes);
     p.boxes_at = nodes_bytes(n_tiles);
@@ -259,7 +266,7 @@ int cluster_prepare(const rsi_stage& st, const double* ks, float gate_ratio, con
     a.nodes = extra;
     a.boxes = extra + p.boxes_at;
     a.gate = reinterpret_cast<StageGate*>(extra + p.extra_bytes - 256);
-    a.gate_ratio = gate_ratio;
+    a.gate_ratio = gate_ratio * p.gain;
     a.weight = kClusterWeight / p.fill;
     a.status = status;
     for (int f = 0; f < p.nf; ++f) {
