@@ -179,14 +179,16 @@ size_t nodes_bytes(int n_tiles) {
 // about 40 us more than the direct kernel's, and 6e8 pairs take that kernel
 // 0.45 ms.  A piston's clusters are small beside the distance and nearly always
 // taken; an interface's may not be, so its sums have to be longer, and those of
-// several frequencies, whose direct sum is shared, three times as long (9e8 and
-// 7.8e8 pairs at three frequencies: 2.25 and 1.5 ms either way, less the 40 us);
+// several frequencies, whose direct sum is shared, two or three times as long (9e8
+// and 7.8e8 pairs at three frequencies: no faster, and 40 us lost);
 // a ray costs the direct kernel 7 times a stage's pair (16384 x 256 x 128:
 // 2.32 -> 1.81 ms, 9001 x 101 x 77: 0.55 -> 1.29 ms).  Per-point normals turn within a
 // tile on every curved surface, where the direct sum would be taken anyway.
 bool cluster_plan(int kind, int normals, int nf, int64_t n_src, int64_t n_tgt, int S, int splits, int max_auto_splits,
                   ClusterPlan& p) {
-    const double least = kind == RSI_TIMING_RAYTRACE ? 3e8 : (kind == RSI_STAGE_PISTON ? 6e8 : 1e9) * (nf > 1 ? 3.0 : 1.0);
+    const double least = kind == RSI_TIMING_RAYTRACE ? 3e8
+                         : kind == RSI_STAGE_PISTON   ? (nf > 1 ? 1e9 : 5e8)
+                                                      : (nf > 1 ? 3e9 : 1e9);
     if (n_src < 8192 || n_tgt < 4096 || double(n_src) * double(n_tgt) < least) return false;
     if (kind == RSI_STAGE_RSI && base_normals(normals) != RSI_NORMALS_Z) return false;
     const int n_tiles = int((n_src + S - 1) / S);
