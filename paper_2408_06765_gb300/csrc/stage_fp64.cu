@@ -1,10 +1,15 @@
 // stage_fp64.cu -- double-precision source x target kernel (steps a3, a5),
 // the path for runs validated at 1e-5 against the FP64 oracle.  Same tiling
-// and bulk-copy pipeline as the FP32C kernel; per pair it evaluates the
-// paper's terms directly in FP64 with Neumaier-compensated accumulation.
+// and bulk-copy pipeline as the FP32C kernel; the paper's terms with an FP64
+// phase and 48-bit amplitudes (stage_fp64_body.cuh), summed in pairs of floats
+// over 32 terms and in doubles with Neumaier compensation over those.
+// 2^12 x 2^12 pairs of a piston stage: 2.08 ms with every operation in doubles
+// (75 of the FP64 pipe per pair, 98 % of the time), 0.50 ms now, of which the
+// pipe's 12 operations take 0.35; of an interface stage 2.37 and 0.50 (0.60 with
+// per-point normals, 15 operations).
 #include <math.h>
 
-#include "stage.cuh"
+#include "stage_fp64_body.cuh"
 
 namespace {
 
@@ -22,9 +27,13 @@ __device__ __forceinline__ void neu_add(Neu& a, double v) {
     a.s = t;
 }
 
+using namespace rsi_fp64;
+__device__ const Tab kTab = make_tab();
+
 template <int KIND, int NORM>
 __global__ void __launch_bounds__(kThreads)
     stage_fp64_kernel(StageArgs a) {
+    __shared__ TabEntry tab[kTabSize];
     extern __shared__ __align__(128) uint8_t smem[];
     const int tid = threadIdx.x;
     const int split = blockIdx.y;
@@ -37,7 +46,8 @@ __global__ void __launch_bounds__(kThreads)
     const int64_t j_raw = int64_t(blockIdx.x) * kThreads + tid;
     const int64_t j = j_raw < a.n_tgt ? j_raw : a.n_tgt - 1;
     const double qx = a.tgt.x[j], qy = a.tgt.y[j], qz = a.tgt.z[j];
-    const double k = a.k;
+    for (int i = tid; i < kTabSize; i += kThreads) tab[i] = kTab.e[i];
+    const Wave w = make_wave(a.k);
 
     if (tid == 0) {
         for (int s = 0; s < RSI_PIPE_STAGES; ++s) mbar_init(smem_u32(&bars[s]), 1);
@@ -63,29 +73,32 @@ __global__ void __launch_bounds__(kThreads)
             failed_at = it;
             break;
         }
-        const double* rec = reinterpret_cast<const double*>(smem + buf * a.tile_bytes + RSI_TILE_HDR_BYTES);
-        for (int i = 0; i < a.S; ++i) {
-            const double* r = rec + 8 * i;
-            const double dx = qx - r[0], dy = qy - r[1], dz = qz - r[2];
-            const double r2 = dx * dx + dy * dy + dz * dz;
-            if (!(r2 >= 1e-24)) continue;  // pairs closer than 1e-12 m contribute nothing
-            const double rr = sqrt(r2);
-            const double ir = 1.0 / rr;
-            double s, c;
-            sincos(k * rr, &s, &c);
-            if (KIND == RSI_STAGE_PISTON) {
-                const double amp = r[3] * ir;  // -v0 w / (2 pi r)
-                neu_add(re, amp * c);
-                neu_add(im, amp * s);
-            } else {
-                const double nd = (NORM == RSI_NORMALS_Z) ? dz : (r[5] * dx + r[6] * dy + r[7] * dz);
-                const double h = nd * ir * ir;  // cos(theta) / r
-                // B (ik - 1/r) e^{ikr} cos(theta) / r,  B = -w sigma / (2 pi)
-                const double vr = -ir * r[3] - k * r[4];
-                const double vi = -ir * r[4] + k * r[3];
-                neu_add(re, h * (vr * c - vi * s));
-                neu_add(im, h * (vr * s + vi * c));
+        const double scale = *reinterpret_cast<const double*>(smem + buf * a.tile_bytes);
+        const Record* rec = reinterpret_cast<const Record*>(smem + buf * a.tile_bytes + RSI_TILE_HDR_BYTES);
+        for (int i0 = 0; i0 < a.S; i0 += 32) {
+            DF sr = {0.0f, 0.0f}, si = {0.0f, 0.0f};
+#pragma unroll 1
+            for (int i = i0; i < i0 + 32; ++i) {
+                const Record& r = rec[i];
+                const double dx = qx - r.x, dy = qy - r.y, dz = qz - r.z;
+                const double r2 = dx * dx + dy * dy + dz * dz;
+                const double nd = (KIND == RSI_STAGE_PISTON) ? 0.0
+                                  : (NORM == RSI_NORMALS_Z)  ? dz
+                                                             : (r.nx * dx + r.ny * dy + r.nz * dz);
+                if (in_range(w, r2)) {
+                    DF fr, fi;
+                    fast_term<KIND>(w, r2, nd, r.a, r.b, tab, fr, fi);
+                    sr = df_add(sr, fr);
+                    si = df_add(si, fi);
+                } else {
+                    const double2 v = slow_term<KIND>(w.k, r2, nd, double(r.a.h) + double(r.a.l),
+                                                      double(r.b.h) + double(r.b.l));
+                    neu_add(re, scale * v.x);
+                    neu_add(im, scale * v.y);
+                }
             }
+            neu_add(re, scale * (double(sr.h) + double(sr.l)));
+            neu_add(im, scale * (double(si.h) + double(si.l)));
         }
         __syncthreads();
         if (tid == 0 && it + RSI_PIPE_STAGES < ntile) {
@@ -111,40 +124,68 @@ __global__ void __launch_bounds__(kThreads)
     }
 }
 
-__global__ void prep_fp64_kernel(int kind, int normals, int64_t n_src, PointsView src,
-                                 const double2* __restrict__ sigma, double amp_scale, uint8_t* tiles,
-                                 size_t tile_bytes, int64_t n_slots) {
-    int64_t q = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (q >= n_slots) return;
-    const int S = int((tile_bytes - RSI_TILE_HDR_BYTES) / 64);
-    const int64_t tile = q / S, slot = q - tile * S;
-    double* rec = reinterpret_cast<double*>(tiles + size_t(tile) * tile_bytes + RSI_TILE_HDR_BYTES) + 8 * slot;
-    if (slot == 0) {
-        double* hdr = reinterpret_cast<double*>(tiles + size_t(tile) * tile_bytes);
-        hdr[0] = hdr[1] = hdr[2] = hdr[3] = 0.0;
+// One CTA per tile: its records, with the amplitudes over a power of two near
+// the largest, so that they are floats of full precision whatever their unit.
+constexpr int kPrepThreads = 128;
+__global__ void __launch_bounds__(kPrepThreads)
+    prep_fp64_kernel(int kind, int S, int64_t n_src, PointsView src, const double2* __restrict__ sigma,
+                     double amp_scale, uint8_t* tiles, size_t tile_bytes) {
+    __shared__ int top;
+    uint8_t* tile = tiles + size_t(blockIdx.x) * tile_bytes;
+    Record* rec = reinterpret_cast<Record*>(tile + RSI_TILE_HDR_BYTES);
+    const int64_t first = int64_t(blockIdx.x) * S;
+    auto amplitude = [&](int64_t q, double& a, double& b) {
+        a = b = 0.0;
+        if (q >= n_src) return;
+        a = amp_scale * src.w[q];
+        if (kind == RSI_STAGE_PISTON) return;
+        const double2 sg = sigma[q];
+        b = a * sg.y;
+        a *= sg.x;
+    };
+    if (threadIdx.x == 0) top = 0;
+    __syncthreads();
+    int largest = 0;
+    for (int i = threadIdx.x; i < S; i += kPrepThreads) {
+        double a, b;
+        amplitude(first + i, a, b);
+        largest = max(largest, max(__double2hiint(a) & 0x7fffffff, __double2hiint(b) & 0x7fffffff));
     }
-    if (q < n_src) {
-        rec[0] = src.x[q];
-        rec[1] = src.y[q];
-        rec[2] = src.z[q];
-        if (kind == RSI_STAGE_PISTON) {
-            rec[3] = amp_scale * src.w[q];
-            rec[4] = 0.0;
-        } else {
-            double2 sg = sigma[q];
-            rec[3] = amp_scale * src.w[q] * sg.x;
-            rec[4] = amp_scale * src.w[q] * sg.y;
-        }
-        rec[5] = src.nx[q];
-        rec[6] = src.ny[q];
-        rec[7] = src.nz[q];
-    } else {
-        rec[0] = rec[1] = rec[2] = 4.0;
-        rec[3] = rec[4] = 0.0;
-        rec[5] = rec[6] = 0.0;
-        rec[7] = 1.0;
+    atomicMax(&top, largest);
+    __syncthreads();
+    // 2^e for 2^e <= largest < 2^(e+1); 1 where there is none or it is not finite
+    const int e = top >> 20;
+    const bool usable = e > 0 && e < 0x7ff;
+    const double scale = usable ? __hiloint2double(e << 20, 0) : 1.0;
+    if (threadIdx.x == 0) {
+        double* hdr = reinterpret_cast<double*>(tile);
+        hdr[0] = scale;
+        hdr[1] = hdr[2] = hdr[3] = 0.0;
     }
-    (void)normals;
+    // 2^-e would overflow for the smallest e: in two factors
+    const int e1 = usable ? (1023 - e) / 2 : 0, e2 = usable ? 1023 - e - e1 : 0;
+    const double f1 = __hiloint2double((1023 + e1) << 20, 0), f2 = __hiloint2double((1023 + e2) << 20, 0);
+    auto pair = [&](double v) {
+        v = v * f1 * f2;
+        const float h = float(v);
+        return DF{h, isfinite(h) ? float(v - double(h)) : 0.0f};
+    };
+    for (int i = threadIdx.x; i < S; i += kPrepThreads) {
+        const int64_t q = first + i;
+        Record r;
+        double a, b;
+        amplitude(q, a, b);
+        r.a = pair(a);
+        r.b = pair(b);
+        const bool real = q < n_src;
+        r.x = real ? src.x[q] : 4.0;
+        r.y = real ? src.y[q] : 4.0;
+        r.z = real ? src.z[q] : 4.0;
+        r.nx = real ? src.nx[q] : 0.0;
+        r.ny = real ? src.ny[q] : 0.0;
+        r.nz = real ? src.nz[q] : 1.0;
+        rec[i] = r;
+    }
 }
 
 template <int KIND, int NORM>
@@ -184,18 +225,14 @@ int dispatch(const StageArgs& a, cudaStream_t s, bool occ) {
 
 }  // namespace
 
-size_t fp64_record_bytes() { return 64; }
+size_t fp64_record_bytes() { return sizeof(Record); }
 int fp64_threads() { return kThreads; }
 
 int launch_prep_fp64(const rsi_stage& st, const PointsView& src, int64_t n_src, const double2* sigma, int S,
                      uint8_t* tiles, size_t tile_bytes, int n_tiles, cudaStream_t s) {
     const double amp_scale = stage_amp_scale(st);
-    const int normals = st.kind == RSI_STAGE_RSI ? base_normals(st.normals) : RSI_NORMALS_Z;
-    int64_t n_slots = int64_t(n_tiles) * S;
-    int threads = 256;
-    unsigned blocks = unsigned((n_slots + threads - 1) / threads);
-    prep_fp64_kernel<<<blocks, threads, 0, s>>>(st.kind, normals, n_src, src, sigma, amp_scale, tiles, tile_bytes,
-                                                n_slots);
+    prep_fp64_kernel<<<unsigned(n_tiles), kPrepThreads, 0, s>>>(st.kind, S, n_src, src, sigma, amp_scale, tiles,
+                                                                tile_bytes);
     RSI_CHECK_LAUNCH("prep_fp64_kernel");
     return RSI_OK;
 }
