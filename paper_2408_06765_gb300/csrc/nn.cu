@@ -15,6 +15,10 @@
 //                DSILU      C * silu'(aux)                   -> bf16   (backprop)
 //              and, tcgen05 only, the output layer with the carrier:
 //                CARRIER    scale exp(+-i psi) (C + bias)    -> f32   (inference)
+//                SILU       silu(C + bias)                   -> bf16  (inference:
+//                           without the z that only backprop reads)
+//                HEAD       the columns' share of W_h silu(C + bias) -> f32
+//                           (inference: the last hidden layer and the head)
 //   transpose  bf16 [R x C] -> [C x R]
 //   loss       mean (y - t)^2 and its gradient 2 (y - t)/n  -> bf16
 //   colsum     bias gradients (column sums of a bf16 matrix)
@@ -60,12 +64,18 @@ __device__ __forceinline__ void mma_bf16(float* c, const uint32_t* a, const uint
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-// logistic sigmoid with the fast reciprocal division (a few ulp; the results
-// are rounded to bf16): no IEEE division and its slow-path branch in the
-// epilogue of every hidden layer.  Past z = -87 exp(-z) is infinite and the
-// quotient the limit 0.
-__device__ __forceinline__ float sigmoidf_(float z) { return __fdividef(1.0f, 1.0f + __expf(-z)); }
+// logistic sigmoid with the hardware's power of two and reciprocal (a few ulp; the
+// results are rounded to bf16), each flushing what lies below 2^-126 to 0, which
+// 1 + exp(-z) does not notice and the quotient reaches as its limit past z = -87:
+// 4 instructions, where __fdividef and __expf guard those ranges with 6 more.
+__device__ __forceinline__ float sigmoidf_(float z) {
+    float e, r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(__fmul_rn(z, -1.4426950408889634f)));  // log2(e)
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__fadd_rn(1.0f, e)));
+    return r;
+}
 __device__ __forceinline__ float silu_(float z) { return z * sigmoidf_(z); }
+__device__ __forceinline__ float bf16_silu_(float z) { return __bfloat162float(__float2bfloat16_rn(silu_(z))); }
 __device__ __forceinline__ float dsilu_(float z) {
     float s = sigmoidf_(z);
     return s * (1.0f + z * (1.0f - s));
@@ -335,6 +345,11 @@ __global__ void carrier_rows_kernel(CarrierArgs ca, int M, float4* __restrict__ 
     rows[2 * b + 1] = make_float4(r.wh, r.wl, r.rc, r.rs);
 }
 
+template <int EPI>
+constexpr bool kF32Out = EPI == 0 || EPI == 1 || EPI == 3;  // through tmC
+template <int EPI>
+constexpr bool kBf16Out = EPI == 1 || EPI == 2 || EPI == 4;  // through tmH
+
 template <int TBN>
 struct TcCfg {
     static constexpr uint32_t B_BYTES = TBN * TC_BK * 2;
@@ -367,7 +382,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                    const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmH, int M, int N,
                    int K, int layout, const float* __restrict__ bias, const float* __restrict__ aux, int kts,
-                   int splits, CarrierArgs car, int* status) {
+                   int splits, CarrierArgs car, float* outy, int* status) {
     // layout bit 0: A is stored [K x M] (MN-major), bit 1: B is stored [K x N]
     const bool a_mn = layout & 1, b_mn = layout & 2;
     // outputs leave by TMA stores: f32 (F32, BIAS_SILU's z, split-K partial
@@ -403,8 +418,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     if (tid == 64) {
         rsi_umma::prefetch_tmap(&tmA);
         rsi_umma::prefetch_tmap(&tmB);
-        if (EPI != 2 || splits > 1) rsi_umma::prefetch_tmap(&tmC);
-        if ((EPI == 1 || EPI == 2) && splits == 1) rsi_umma::prefetch_tmap(&tmH);  // bf16 outputs only
+        if (kF32Out<EPI> || splits > 1) rsi_umma::prefetch_tmap(&tmC);
+        if (kBf16Out<EPI> && splits == 1) rsi_umma::prefetch_tmap(&tmH);
     }
     rsi_umma::fence_before_sync();
     __syncthreads();
@@ -515,8 +530,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             rsi_umma::fence_after_sync();
             const uint32_t sbuf = smem_u32(buf);  // 1024-byte aligned: 32 rows of 128 B, 128-byte swizzle atoms
             const int row0 = T.m0 + q * 32;       // this warp's first output row; lane = row - row0
-#pragma unroll 1
-            for (int cb = h * (TBN / 2); cb < (h + 1) * (TBN / 2); cb += 32) {
+            float y0 = 0.0f, y1 = 0.0f, y2 = 0.0f;  // EPI 5
+            // a block's accumulators are read while the block before is worked on
+            const uint32_t acc0 = tmem + (uint32_t(q * 32) << 16) + uint32_t(acc * TBN + h * (TBN / 2));
+            uint32_t rv[2][32];
+            rsi_umma::ld_32x32b_x32(acc0, rv[0]);
+#pragma unroll
+            for (int ib = 0; ib < TBN / 64; ++ib) {
+                const int cb = h * (TBN / 2) + 32 * ib;
                 const int col0 = T.n0 + cb;
                 float a[32];
                 if (EPI == 2 && splits == 1) {  // the pre-activations this row's outputs need, ahead of the TMEM read
@@ -529,13 +550,17 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                         a[4 * i + 3] = z.w;
                     }
                 }
-                float v[32];
-                rsi_umma::ld_32x32b_x32(tmem + (uint32_t(q * 32) << 16) + uint32_t(acc * TBN + cb), v);
-                if (cb + 32 == (h + 1) * (TBN / 2)) {  // this warp's last read of the accumulator
+                rsi_umma::ld_wait(rv[ib & 1]);
+                if (ib + 1 < TBN / 64) {
+                    rsi_umma::ld_32x32b_x32(acc0 + 32u * (ib + 1), rv[(ib + 1) & 1]);
+                } else {  // this warp's last read of the accumulator
                     rsi_umma::fence_before_sync();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(smem_u32(&acc_empty[acc]));
                 }
+                float v[32];
+#pragma unroll
+                for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(rv[ib & 1][i]);
                 if (add_bias) {
                     const int src = (cb - h * (TBN / 2)) / 4;  // the lane holding columns col0 .. col0 + 3
 #pragma unroll
@@ -576,7 +601,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                         }
                     }
                 }
-                if (EPI != 2 || splits > 1) {  // f32 block: output, z, or partial sums of split T.z
+                if (kF32Out<EPI> || splits > 1) {  // f32 block: output, z, or partial sums of split T.z
                     if (lane == 0) rsi_umma::bulk_wait_read0();  // the previous block has left buf
                     __syncwarp();
 #pragma unroll
@@ -590,29 +615,53 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                         rsi_umma::bulk_commit();
                     }
                 }
-                if ((EPI == 1 || EPI == 2) && splits == 1) {  // bf16 block (dense 64-byte rows): silu(z) or C * silu'(aux)
+                if (EPI == 5) {  // three dot products of this row's outputs, rounded as the bf16 layer would be
+                    const float* wh = aux + col0;
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const float4 w0 = __ldg(reinterpret_cast<const float4*>(wh) + i),
+                                     w1 = __ldg(reinterpret_cast<const float4*>(wh + N) + i),
+                                     w2 = __ldg(reinterpret_cast<const float4*>(wh + 2 * N) + i);
+                        const float x0 = bf16_silu_(v[4 * i]), x1 = bf16_silu_(v[4 * i + 1]),
+                                    x2 = bf16_silu_(v[4 * i + 2]), x3 = bf16_silu_(v[4 * i + 3]);
+                        y0 = fmaf(w0.x, x0, fmaf(w0.y, x1, fmaf(w0.z, x2, fmaf(w0.w, x3, y0))));
+                        y1 = fmaf(w1.x, x0, fmaf(w1.y, x1, fmaf(w1.z, x2, fmaf(w1.w, x3, y1))));
+                        y2 = fmaf(w2.x, x0, fmaf(w2.y, x1, fmaf(w2.z, x2, fmaf(w2.w, x3, y2))));
+                    }
+                }
+                if (kBf16Out<EPI> && splits == 1) {  // bf16 block (dense 64-byte rows): silu(z) or C * silu'(aux)
                     uint32_t hw[16];
 #pragma unroll
                     for (int j = 0; j < 16; ++j) {
-                        const float x0 = EPI == 1 ? silu_(v[2 * j]) : v[2 * j] * dsilu_(a[2 * j]);
-                        const float x1 = EPI == 1 ? silu_(v[2 * j + 1]) : v[2 * j + 1] * dsilu_(a[2 * j + 1]);
+                        const float x0 = EPI != 2 ? silu_(v[2 * j]) : v[2 * j] * dsilu_(a[2 * j]);
+                        const float x1 = EPI != 2 ? silu_(v[2 * j + 1]) : v[2 * j + 1] * dsilu_(a[2 * j + 1]);
                         __nv_bfloat162 p2 = __floats2bfloat162_rn(x0, x1);
                         hw[j] = *reinterpret_cast<uint32_t*>(&p2);
                     }
-                    if (lane == 0) rsi_umma::bulk_wait_read0();
+                    // without f32 output the two halves of buf take turns
+                    uint8_t* hb = reinterpret_cast<uint8_t*>(buf) + (EPI != 1 && ((tc * (TBN / 64) + ib) & 1) ? 2048 : 0);
+                    if (lane == 0) {
+                        if (EPI == 1)
+                            rsi_umma::bulk_wait_read0();
+                        else
+                            rsi_umma::bulk_wait_read1();
+                    }
                     __syncwarp();
 #pragma unroll
                     for (int c = 0; c < 4; ++c)
-                        *reinterpret_cast<uint4*>(reinterpret_cast<uint8_t*>(buf) + lane * 64 + 16 * c) =
+                        *reinterpret_cast<uint4*>(hb + lane * 64 + 16 * c) =
                             make_uint4(hw[4 * c], hw[4 * c + 1], hw[4 * c + 2], hw[4 * c + 3]);
                     rsi_umma::fence_proxy_async_smem();
                     __syncwarp();
                     if (lane == 0) {
-                        rsi_umma::tma_store_2d(&tmH, col0, row0, sbuf);
+                        rsi_umma::tma_store_2d(&tmH, col0, row0, smem_u32(hb));
                         rsi_umma::bulk_commit();
                     }
                 }
             }
+            if (EPI == 5)  // [column half of a tile][row]
+                reinterpret_cast<float4*>(outy)[size_t(T.n0 / (TBN / 2) + h) * M + row0 + lane] =
+                    make_float4(y0, y1, y2, 0.0f);
         }
     }
     if (warp >= 2 && lane == 0) rsi_umma::bulk_wait0();  // this warp's stores are complete
@@ -932,27 +981,36 @@ int gemm_tc_launch_bn(const bf16* A, const bf16* B, int M, int N, int K, int lay
     splits = (kt + kts - 1) / kts;
     memset(&tc, 0, sizeof(tc));
     memset(&th, 0, sizeof(th));
-    if (EPI != 2 || splits > 1) {  // f32 blocks of 32 x 32: the output, z, or the partial sums
+    if (kF32Out<EPI> || splits > 1) {  // f32 blocks of 32 x 32: the output, z, or the partial sums
         rc = make_tmap(&tc, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, splits > 1 ? static_cast<const void*>(work) : outf,
                        int64_t(splits) * M, N, 32, 32);
         if (rc) return rc;
     }
-    if ((EPI == 1 || EPI == 2) && splits == 1) {  // bf16 blocks of 32 x 32, dense 64-byte rows in shared memory
+    if (kBf16Out<EPI> && splits == 1) {  // bf16 blocks of 32 x 32, dense 64-byte rows in shared memory
         rc = make_tmap(&th, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, outh, M, N, 32, 32, CU_TENSOR_MAP_SWIZZLE_NONE);
         if (rc) return rc;
     }
     const int tiles = (M / TC_BM) * (N / TBN) * splits;
     const int grid = std::min(tiles, sm_count());
     gemm_tc_kernel<EPI, TBN><<<grid, TC_THREADS, C::SMEM, s>>>(ta, tb, tc, th, M, N, K, layout, bias, aux, kts,
-                                                               splits, car, status);
+                                                               splits, car, outf, status);
     RSI_CHECK_LAUNCH("gemm_tc_kernel");
-    if (splits > 1) {
-        int64_t pairs = int64_t(M) * N / 2;
-        splitk_reduce_kernel<EPI><<<unsigned((pairs + 255) / 256), 256, 0, s>>>(work, splits, M, N, bias, aux,
-                                                                                 outf, outh);
-        RSI_CHECK_LAUNCH("splitk_reduce_kernel");
-    }
+    if constexpr (EPI < 3)
+        if (splits > 1) {
+            int64_t pairs = int64_t(M) * N / 2;
+            splitk_reduce_kernel<EPI><<<unsigned((pairs + 255) / 256), 256, 0, s>>>(work, splits, M, N, bias, aux,
+                                                                                     outf, outh);
+            RSI_CHECK_LAUNCH("splitk_reduce_kernel");
+        }
     return RSI_OK;
+}
+
+// the output tile's width: see gemm_tc_launch
+int tc_tile_width(int M, int N, int K, int splits) {
+    const int64_t rows = M / TC_BM, sms = sm_count();
+    const int kt = K / TC_BK, units = (kt + (kt + splits - 1) / splits - 1) / ((kt + splits - 1) / splits);
+    if (N % 256 == 0 && rows * (N / 256) * units >= sms) return 256;
+    return N % 128 == 0 && rows * (N / 128) * units >= sms ? 128 : 64;
 }
 
 template <int EPI>
@@ -963,12 +1021,9 @@ int gemm_tc_launch(const bf16* A, const bf16* B, int M, int N, int K, int layout
     // narrowest.  Small GEMMs (the hidden layers at batch 256) are latency-
     // bound: narrower tiles spread them over more SMs and shorten each CTA's
     // main loop and epilogue.
-    const int64_t rows = M / TC_BM, sms = sm_count();
-    const int kt = K / TC_BK, units = (kt + (kt + splits - 1) / splits - 1) / ((kt + splits - 1) / splits);
-    if (N % 256 == 0 && rows * (N / 256) * units >= sms)
-        return gemm_tc_launch_bn<EPI, 256>(A, B, M, N, K, layout, bias, aux, outf, outh, splits, work, s, car);
-    if (N % 128 == 0 && rows * (N / 128) * units >= sms)
-        return gemm_tc_launch_bn<EPI, 128>(A, B, M, N, K, layout, bias, aux, outf, outh, splits, work, s, car);
+    const int w = tc_tile_width(M, N, K, splits);
+    if (w == 256) return gemm_tc_launch_bn<EPI, 256>(A, B, M, N, K, layout, bias, aux, outf, outh, splits, work, s, car);
+    if (w == 128) return gemm_tc_launch_bn<EPI, 128>(A, B, M, N, K, layout, bias, aux, outf, outh, splits, work, s, car);
     return gemm_tc_launch_bn<EPI, 64>(A, B, M, N, K, layout, bias, aux, outf, outh, splits, work, s, car);
 }
 
@@ -1056,6 +1111,20 @@ extern "C" int rsi_nn_gemm(int32_t epilogue, int32_t engine, int32_t layout, con
         default:
             return rsi_fail(RSI_E_INVAL, "rsi_nn_gemm: unknown epilogue %d", epilogue);
     }
+}
+
+// Hidden layers of inference on the tcgen05 engine (nn_net.cu); the caller has
+// checked the sizes and alignments (its own layout of the activations).
+int rsi_nn_layer_silu(const void* A, const void* B, int M, int N, int K, const float* bias, void* out_bf16,
+                      cudaStream_t s) {
+    return gemm_tc_launch<4>(static_cast<const bf16*>(A), static_cast<const bf16*>(B), M, N, K, 0, bias, nullptr,
+                             nullptr, static_cast<bf16*>(out_bf16), 1, nullptr, s);
+}
+int rsi_nn_layer_head_parts(int M, int N, int K) { return 2 * N / tc_tile_width(M, N, K, 1); }
+int rsi_nn_layer_head(const void* A, const void* B, int M, int N, int K, const float* bias, const float* head,
+                      float* parts, cudaStream_t s) {
+    return gemm_tc_launch<5>(static_cast<const bf16*>(A), static_cast<const bf16*>(B), M, N, K, 0, bias, head, parts,
+                             nullptr, 1, nullptr, s);
 }
 
 extern "C" int rsi_nn_gemm_carrier(const void* A, const void* B, int32_t M, int32_t N, int32_t K, const float* bias,

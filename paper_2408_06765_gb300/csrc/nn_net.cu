@@ -147,34 +147,8 @@ __device__ __forceinline__ uint64_t splitmix64(uint64_t s) {
     return z ^ (z >> 31);
 }
 
-// One warp per row: the (field, pixel) pair, the 9 inputs c, then columns
-// [sin(pi B c) | cos(pi B c) | c, 0...] with the Fourier columns spread over
-// the lanes (consecutive lanes write consecutive columns).
-__global__ void __launch_bounds__(256) rows_kernel(RowK k, const double* __restrict__ params, int64_t n_fields,
-                                                   int mode, uint64_t seed, const uint64_t* __restrict__ seed_dev,
-                                                   int64_t first, const float* __restrict__ targets,
-                                                   const float* __restrict__ log_rms, int R, bf16* __restrict__ h0,
-                                                   float4* __restrict__ t_rows) {
-    extern __shared__ float sB[];  // [F][9]
-    for (int e = threadIdx.x; e < k.F * RSI_NN_IN; e += blockDim.x) sB[e] = k.fmat[e];
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
-    const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (r >= R) return;
-    int64_t b, q;
-    if (mode == RSI_NN_ROWS_RANDOM) {
-        const uint64_t sd = seed_dev ? *seed_dev : seed;
-        const uint64_t u = splitmix64(sd + 0x9E3779B97F4A7C15ull * uint64_t(r + 1));
-        b = int64_t((uint64_t(uint32_t(u >> 32)) * uint64_t(n_fields)) >> 32);
-        q = int64_t((uint64_t(uint32_t(u)) * uint64_t(k.npix)) >> 32);
-    } else {
-        int64_t g = first + r;
-        const int64_t last = n_fields * int64_t(k.npix) - 1;
-        g = g < last ? g : last;
-        b = g / k.npix;
-        q = g - b * k.npix;
-    }
-    const double* p = params + 5 * b;
+// the 9 inputs of pixel q of a field (params p)
+__device__ __forceinline__ void row_inputs(const RowK& k, const double* __restrict__ p, int64_t q, float* c) {
     const float tilt = float(p[1]), L = float(p[2]), f = float(p[3]), d = float(p[4]);
     const int i = int(q % k.nx), j = int(q / k.nx);
     const float sg = tilt < 0.0f ? -1.0f : 1.0f;
@@ -186,7 +160,6 @@ __global__ void __launch_bounds__(256) rows_kernel(RowK k, const double* __restr
     const float cth = sqrtf(fmaxf(0.0f, 1.0f - sth * sth));
     const float s = x * sth + z * cth, t = x * cth - z * sth;
     const float fq = k.a2_over_c1 * f / (L + k.c21 * fmaxf(s, 0.0f));
-    float c[RSI_NN_IN];
     c[0] = (a1 - k.lo[0]) * k.inv_span[0] - 1.0f;
     c[1] = (L - k.lo[1]) * k.inv_span[1] - 1.0f;
     c[2] = (f - k.lo[2]) * k.inv_span[2] - 1.0f;
@@ -196,21 +169,83 @@ __global__ void __launch_bounds__(256) rows_kernel(RowK k, const double* __restr
     c[6] = s * k.inv_S0;
     c[7] = t * k.inv_S0;
     c[8] = logf(fq);
-    bf16* row = h0 + size_t(r) * k.K0;
-    for (int fi = lane; fi < k.F; fi += 32) {
-        const float* Bf = sB + fi * RSI_NN_IN;
-        float arg = 0.0f;
+}
+
+// One warp per kRowsPerWarp rows: each lane finds one row's (field, pixel) pair
+// and its 9 inputs c; then, row by row with c handed round by shuffles, the
+// columns [sin(pi B c) | cos(pi B c) | c, 0...].  A lane keeps its pairs of
+// neighbouring Fourier rows (64 i + 2 lane, + 1) in registers for all rows and
+// stores them as one word, so that a row costs the 248 sincospif, 20 us for 65536
+// rows where the bytes take 10 us; with the inputs formed by every lane of a
+// warp per row, B read from shared memory and 2-byte stores it took 62 us.
+constexpr int kRowsPerWarp = 16;
+constexpr int kPairs = 4;  // per lane: 256 Fourier rows per CTA row (blockIdx.y)
+__global__ void __launch_bounds__(256) rows_kernel(RowK k, const double* __restrict__ params, int64_t n_fields,
+                                                   int mode, uint64_t seed, const uint64_t* __restrict__ seed_dev,
+                                                   int64_t first, const float* __restrict__ targets,
+                                                   const float* __restrict__ log_rms, int R, bf16* __restrict__ h0,
+                                                   float4* __restrict__ t_rows) {
+    const int lane = threadIdx.x & 31;
+    const int r0 = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * kRowsPerWarp;
+    const int f0 = blockIdx.y * 64 * kPairs;
+    if (r0 >= R) return;
+    float B[kPairs][2][RSI_NN_IN];
 #pragma unroll
-        for (int m = 0; m < RSI_NN_IN; ++m) arg = fmaf(Bf[m], c[m], arg);
-        float sn, cs;
-        sincospif(arg, &sn, &cs);
-        row[fi] = __float2bfloat16_rn(sn);
-        row[k.F + fi] = __float2bfloat16_rn(cs);
+    for (int n = 0; n < kPairs; ++n)
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+#pragma unroll
+            for (int m = 0; m < RSI_NN_IN; ++m) {
+                const int fi = f0 + 64 * n + 2 * lane + e;
+                B[n][e][m] = fi < k.F ? k.fmat[fi * RSI_NN_IN + m] : 0.0f;
+            }
+    float mine[RSI_NN_IN];
+    {
+        const int r = min(r0 + lane % kRowsPerWarp, R - 1);
+        int64_t b, q;
+        if (mode == RSI_NN_ROWS_RANDOM) {
+            const uint64_t sd = seed_dev ? *seed_dev : seed;
+            const uint64_t u = splitmix64(sd + 0x9E3779B97F4A7C15ull * uint64_t(r + 1));
+            b = int64_t((uint64_t(uint32_t(u >> 32)) * uint64_t(n_fields)) >> 32);
+            q = int64_t((uint64_t(uint32_t(u)) * uint64_t(k.npix)) >> 32);
+        } else {
+            int64_t g = first + r;
+            const int64_t last = n_fields * int64_t(k.npix) - 1;
+            g = g < last ? g : last;
+            b = g / k.npix;
+            q = g - b * k.npix;
+        }
+        row_inputs(k, params + 5 * b, q, mine);
+        if (targets && lane < kRowsPerWarp && r0 + lane < R) {
+            const float* tg = targets + 2 * (b * int64_t(k.npix) + q);
+            t_rows[r] = make_float4(tg[0], tg[1], log_rms[b], 0.0f);
+        }
     }
-    if (lane < kRaw) row[2 * k.F + lane] = __float2bfloat16_rn(lane < RSI_NN_IN ? c[lane] : 0.0f);
-    if (targets && lane == 0) {
-        const float* tg = targets + 2 * (b * int64_t(k.npix) + q);
-        t_rows[r] = make_float4(tg[0], tg[1], log_rms[b], 0.0f);
+#pragma unroll 1
+    for (int i = 0; i < kRowsPerWarp && r0 + i < R; ++i) {
+        float c[RSI_NN_IN], raw = 0.0f;
+#pragma unroll
+        for (int m = 0; m < RSI_NN_IN; ++m) {
+            c[m] = __shfl_sync(0xffffffffu, mine[m], i);
+            raw = lane == m ? c[m] : raw;
+        }
+        bf16* row = h0 + size_t(r0 + i) * k.K0;
+#pragma unroll
+        for (int n = 0; n < kPairs; ++n) {
+            const int fi = f0 + 64 * n + 2 * lane;
+            if (fi >= k.F) continue;
+            float sn[2], cs[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                float arg = 0.0f;
+#pragma unroll
+                for (int m = 0; m < RSI_NN_IN; ++m) arg = fmaf(B[n][e][m], c[m], arg);
+                sincospif(arg, &sn[e], &cs[e]);
+            }
+            *reinterpret_cast<__nv_bfloat162*>(row + fi) = __floats2bfloat162_rn(sn[0], sn[1]);
+            *reinterpret_cast<__nv_bfloat162*>(row + k.F + fi) = __floats2bfloat162_rn(cs[0], cs[1]);
+        }
+        if (lane < kRaw && f0 == 0) row[2 * k.F + lane] = __float2bfloat16_rn(raw);
     }
 }
 
@@ -387,23 +422,58 @@ __global__ void __launch_bounds__(256) colsum_part_kernel(const bf16* __restrict
     part[size_t(blockIdx.y) * cols + c + 1] = s1;
 }
 
-// per field (one CTA): the mean of the log-RMS outputs over its pixels, then
-// exp(mean) (re, im) interleaved for the carrier pass
-__global__ void __launch_bounds__(256) assemble_kernel(const float4* __restrict__ y, int npix,
-                                                       float2* __restrict__ env) {
+// The head's outputs of a chunk of a field's pixels from the partial sums of the
+// last layer's columns ([part][R], in order, then the bias), and the chunk's sum of
+// the log-RMS outputs.  Field blockIdx.x, chunk blockIdx.y; chunks of 1024
+// pixels keep every SM busy where one CTA per field took 48 us for 4 fields.
+constexpr int kChunk = 1024;
+__device__ __forceinline__ double block_sum(double s) {
     __shared__ double red[256];
-    const float4* yb = y + size_t(blockIdx.x) * npix;
-    double s = 0.0;
-    for (int p = threadIdx.x; p < npix; p += blockDim.x) s += double(yb[p].z);
     red[threadIdx.x] = s;
     for (int st = 128; st > 0; st >>= 1) {
         __syncthreads();
         if (threadIdx.x < st) red[threadIdx.x] += red[threadIdx.x + st];
     }
     __syncthreads();
-    const float amp = float(exp(red[0] / double(npix)));
+    return red[0];
+}
+__global__ void __launch_bounds__(256) head_sum_kernel(const float4* __restrict__ parts, int n_parts, int R,
+                                                       const float* __restrict__ bh, int npix, float4* __restrict__ y,
+                                                       double* __restrict__ chunk_sum) {
+    const float b0 = bh[0], b1 = bh[1], b2 = bh[2];
+    double s = 0.0;
+    for (int p = blockIdx.y * kChunk + threadIdx.x; p < min(npix, (int(blockIdx.y) + 1) * kChunk); p += 256) {
+        const size_t r = size_t(blockIdx.x) * npix + p;
+        float4 v = parts[r];
+        for (int i = 1; i < n_parts; ++i) {
+            const float4 w = parts[size_t(i) * R + r];
+            v.x += w.x, v.y += w.y, v.z += w.z;
+        }
+        v = make_float4(v.x + b0, v.y + b1, v.z + b2, 0.0f);
+        y[r] = v;
+        s += double(v.z);
+    }
+    s = block_sum(s);
+    if (threadIdx.x == 0) chunk_sum[size_t(blockIdx.x) * gridDim.y + blockIdx.y] = s;
+}
+__global__ void __launch_bounds__(256) log_rms_kernel(const float4* __restrict__ y, int npix,
+                                                      double* __restrict__ chunk_sum) {
+    double s = 0.0;
+    for (int p = blockIdx.y * kChunk + threadIdx.x; p < min(npix, (int(blockIdx.y) + 1) * kChunk); p += 256)
+        s += double(y[size_t(blockIdx.x) * npix + p].z);
+    s = block_sum(s);
+    if (threadIdx.x == 0) chunk_sum[size_t(blockIdx.x) * gridDim.y + blockIdx.y] = s;
+}
+// exp(mean of the log-RMS outputs over the field) (re, im), interleaved for the carrier pass
+__global__ void __launch_bounds__(256) assemble_kernel(const float4* __restrict__ y, int npix,
+                                                       const double* __restrict__ chunk_sum, float2* __restrict__ env) {
+    double s = 0.0;
+    for (int c = threadIdx.x; c < int(gridDim.y); c += 256) s += chunk_sum[size_t(blockIdx.x) * gridDim.y + c];
+    const float amp = float(exp(block_sum(s) / double(npix)));
+    const float4* yb = y + size_t(blockIdx.x) * npix;
     float2* eb = env + size_t(blockIdx.x) * npix;
-    for (int p = threadIdx.x; p < npix; p += blockDim.x) eb[p] = make_float2(amp * yb[p].x, amp * yb[p].y);
+    for (int p = blockIdx.y * kChunk + threadIdx.x; p < min(npix, (int(blockIdx.y) + 1) * kChunk); p += 256)
+        eb[p] = make_float2(amp * yb[p].x, amp * yb[p].y);
 }
 
 // training targets of one field (one CTA): the demodulated image over its RMS
@@ -500,12 +570,12 @@ extern "C" int rsi_nn_rows(const rsi_nn_net* net, const double* params, int64_t 
         return rsi_fail(RSI_E_INVAL, "rsi_nn_rows: first row outside the fields' pixels");
     if (bool(targets) != bool(log_rms)) return rsi_fail(RSI_E_INVAL, "rsi_nn_rows: targets need log_rms");
     const RowK k = row_consts(*net, d);
-    const int warps = 8;
-    const size_t smem = size_t(d.F) * RSI_NN_IN * sizeof(float);
-    if (smem > 48 * 1024) return rsi_fail(RSI_E_INVAL, "rsi_nn_rows: n_freq too large");
-    rows_kernel<<<unsigned((d.R + warps - 1) / warps), 32 * warps, smem, static_cast<cudaStream_t>(stream)>>>(
-        k, params, n_fields, mode, seed, seed_dev, first, targets, log_rms, d.R, at<bf16>(act, a.h[0]),
-        at<float4>(act, a.t));
+    if (size_t(d.F) * RSI_NN_IN * sizeof(float) > 48 * 1024)
+        return rsi_fail(RSI_E_INVAL, "rsi_nn_rows: n_freq too large");
+    const int per = 8 * kRowsPerWarp;
+    rows_kernel<<<dim3(unsigned((d.R + per - 1) / per), unsigned((d.F + 64 * kPairs - 1) / (64 * kPairs))), 256, 0,
+                  static_cast<cudaStream_t>(stream)>>>(k, params, n_fields, mode, seed, seed_dev, first, targets, log_rms,
+                                                       d.R, at<bf16>(act, a.h[0]), at<float4>(act, a.t));
     RSI_CHECK_LAUNCH("rows_kernel");
     return RSI_OK;
 }
@@ -617,14 +687,39 @@ extern "C" int rsi_nn_infer(const rsi_nn_net* net, const void* w16, const float*
     if (d.R % d.npix) return rsi_fail(RSI_E_INVAL, "rsi_nn_infer: rows must be a multiple of the window's pixels");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int per = d.R / d.npix;  // fields per chunk
+    const bf16* W16 = static_cast<const bf16*>(w16);
+    // the tcgen05 layers without what only the backward pass reads: no z (134 of
+    // the 268 MB of a layer of 65536 rows), and the head in the last layer's
+    // epilogue, before its outputs leave the SM
+    const bool fused = net->engine == RSI_NN_ENGINE_TCGEN05 &&
+                       ((reinterpret_cast<uintptr_t>(w16) | reinterpret_cast<uintptr_t>(w32)) & 15) == 0;
+    const unsigned chunks = unsigned((d.npix + kChunk - 1) / kChunk);
     for (int f0 = 0; f0 < n_fields; f0 += per) {
         const int nf = std::min(per, n_fields - f0);
         rc = rsi_nn_rows(net, params, n_fields, RSI_NN_ROWS_PIXELS, 0, nullptr, int64_t(f0) * d.npix, nullptr,
                          nullptr, act, act_bytes, stream);
         if (rc != RSI_OK) return rc;
-        rc = hidden_forward(*net, d, a, static_cast<const bf16*>(w16), w32, act, s);
+        double* chunk_sum = at<double>(act, a.part);
+        for (int l = 0; fused && l < d.D && rc == RSI_OK; ++l) {
+            const bf16 *h = at<bf16>(act, a.h[l]), *w = W16 + w_off(d, l);
+            const float* b = w32 + b_off(d, l);
+            rc = l + 1 < d.D ? rsi_nn_layer_silu(h, w, d.R, d.W, in_of(d, l), b, at<bf16>(act, a.h[l + 1]), s)
+                             : rsi_nn_layer_head(h, w, d.R, d.W, in_of(d, l), b, w32 + w_off(d, d.D),
+                                                 at<float>(act, a.z[1]), s);
+        }
+        if (!fused) rc = hidden_forward(*net, d, a, W16, w32, act, s);
         if (rc != RSI_OK) return rc;
-        assemble_kernel<<<unsigned(nf), 256, 0, s>>>(at<float4>(act, a.y), d.npix, at<float2>(act, a.env));
+        const dim3 grid(unsigned(nf), chunks);
+        if (fused) {
+            head_sum_kernel<<<grid, 256, 0, s>>>(at<float4>(act, a.z[1]),
+                                                 rsi_nn_layer_head_parts(d.R, d.W, in_of(d, d.D - 1)), d.R,
+                                                 w32 + b_off(d, d.D), d.npix, at<float4>(act, a.y), chunk_sum);
+            RSI_CHECK_LAUNCH("head_sum_kernel");
+        } else {
+            log_rms_kernel<<<grid, 256, 0, s>>>(at<float4>(act, a.y), d.npix, chunk_sum);
+            RSI_CHECK_LAUNCH("log_rms_kernel");
+        }
+        assemble_kernel<<<grid, 256, 0, s>>>(at<float4>(act, a.y), d.npix, chunk_sum, at<float2>(act, a.env));
         RSI_CHECK_LAUNCH("assemble_kernel");
         rc = rsi_nn_carrier_coeffs(params + 5 * size_t(f0), nf, net->c1, net->c2, carrier + 4 * size_t(f0),
                                    at<float>(act, a.p32), stream);

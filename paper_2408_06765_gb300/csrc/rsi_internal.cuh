@@ -75,6 +75,15 @@ struct PointsView {
 size_t rsi_field_bytes_(int32_t field, int64_t n);
 PointsView rsi_points_view(void* base, int64_t n);
 
+// hidden layers of the surrogate's inference (nn.cu): out = silu(A B^T + bias) in
+// bf16; and, with the head's weights [3][N], `parts` partial sums [part][M] float4
+// of W_h silu(A B^T + bias) instead of the layer
+int rsi_nn_layer_silu(const void* A, const void* B, int M, int N, int K, const float* bias, void* out_bf16,
+                      cudaStream_t s);
+int rsi_nn_layer_head_parts(int M, int N, int K);
+int rsi_nn_layer_head(const void* A, const void* B, int M, int N, int K, const float* bias, const float* head,
+                      float* parts, cudaStream_t s);
+
 // ---------------------------------------------------------------------------
 // double-float (pairs of FP32) arithmetic: error-free transformations of
 // Knuth (TwoSum), Dekker (FastTwoSum) and the FMA-based TwoProduct

@@ -74,6 +74,9 @@ __device__ __forceinline__ void tma_store_2d(const void* tmap, int32_t x, int32_
 }
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 // this thread's bulk stores have finished reading shared memory
+__device__ __forceinline__ void bulk_wait_read1() {  // all but the latest group have been read
+    asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+}
 __device__ __forceinline__ void bulk_wait_read0() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 // this thread's bulk stores are complete
 __device__ __forceinline__ void bulk_wait0() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
@@ -114,22 +117,25 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 // 32 lanes x 32 consecutive 32-bit columns: thread t of the warp gets lane
-// (warp's lane base + t), columns col .. col + 31
-__device__ __forceinline__ void ld_32x32b_x32(uint32_t taddr, float* v) {
-    uint32_t r[32];
+// (warp's lane base + t), columns col .. col + 31.  The load is asynchronous: r
+// holds the values once ld_wait has returned.
+#define RSI_UMMA_R8(c, r, b) \
+    c(r[b]), c(r[b + 1]), c(r[b + 2]), c(r[b + 3]), c(r[b + 4]), c(r[b + 5]), c(r[b + 6]), c(r[b + 7])
+__device__ __forceinline__ void ld_32x32b_x32(uint32_t taddr, uint32_t (&r)[32]) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
         "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : RSI_UMMA_R8("=r", r, 0), RSI_UMMA_R8("=r", r, 8), RSI_UMMA_R8("=r", r, 16), RSI_UMMA_R8("=r", r, 24)
         : "r"(taddr)
         : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
+__device__ __forceinline__ void ld_wait(uint32_t (&r)[32]) {  // every load issued; r passes through, so its uses stay behind
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : RSI_UMMA_R8("+r", r, 0), RSI_UMMA_R8("+r", r, 8), RSI_UMMA_R8("+r", r, 16), RSI_UMMA_R8("+r", r, 24)
+                 :
+                 : "memory");
+}
+#undef RSI_UMMA_R8
 #endif
 
 }  // namespace rsi_umma
