@@ -269,7 +269,8 @@ __global__ void __launch_bounds__(256) head_fwd_kernel(const bf16* __restrict__ 
     }
     const float b0 = bh[0], b1 = bh[1], b2 = bh[2];
     const int warps = gridDim.x * (blockDim.x >> 5);
-    for (int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < R; r += warps) {
+#pragma unroll 2
+    for (int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < R; r += warps) {  // two rows' loads in flight
         const bf16* h = H + size_t(r) * W;
         float a0 = 0.0f, a1 = 0.0f, a2 = 0.0f;
 #pragma unroll
@@ -380,22 +381,27 @@ __global__ void __launch_bounds__(256) head_bwd_kernel(const bf16* __restrict__ 
 }
 
 // sum over chunks of per-chunk partial sums part[chunk][n], in a fixed order:
-// 32 values per CTA, 8 lanes per value each taking every 8th chunk (FP64),
-// the lanes added in lane order.  Values e < n_w go to out_w[e], the next
-// n_b to out_b, a last one (if n > n_w + n_b) times last_scale to *last.
+// 8 values per CTA, 32 lanes per value each taking every 32nd chunk (FP64), the
+// lanes added by halves.  Values e < n_w go to out_w[e], the next n_b to out_b, a
+// last one (if n > n_w + n_b) times last_scale to *last.  The FP64 pipe's 2 lanes
+// per SM bound it: 512 values of 512 chunks took 13.5 us over 16 CTAs of 32
+// values, 6 us (4 of them the launch) over 64.
+constexpr int kSumValues = 8, kSumLanes = 32;
 __global__ void __launch_bounds__(256) chunk_sum_kernel(const float* __restrict__ part, int chunks, int n, int n_w,
                                                         int n_b, float last_scale, float* __restrict__ out_w,
                                                         float* __restrict__ out_b, float* __restrict__ last) {
-    __shared__ double red[8][33];
-    const int e = blockIdx.x * 32 + threadIdx.x;
+    __shared__ double red[kSumLanes][kSumValues + 1];
+    const int e = blockIdx.x * kSumValues + threadIdx.x;
     double acc = 0.0;
     if (e < n)
-        for (int c = threadIdx.y; c < chunks; c += 8) acc += double(part[size_t(c) * n + e]);
+        for (int c = threadIdx.y; c < chunks; c += kSumLanes) acc += double(part[size_t(c) * n + e]);
     red[threadIdx.y][threadIdx.x] = acc;
-    __syncthreads();
+    for (int st = kSumLanes / 2; st > 0; st >>= 1) {
+        __syncthreads();
+        if (threadIdx.y < st) red[threadIdx.y][threadIdx.x] += red[threadIdx.y + st][threadIdx.x];
+    }
     if (threadIdx.y != 0 || e >= n) return;
-    double t = 0.0;
-    for (int k = 0; k < 8; ++k) t += red[k][threadIdx.x];
+    const double t = red[0][threadIdx.x];
     if (e < n_w)
         out_w[e] = float(t);
     else if (e < n_w + n_b)
@@ -617,7 +623,7 @@ extern "C" int rsi_nn_backward(const rsi_nn_net* net, const void* w16, const flo
         w32 + w_off(d, d.D), g, at<bf16>(act, a.dz[cur]), at<float>(act, a.part));
     RSI_CHECK_LAUNCH("head_bwd_kernel");
     const int n_part = kHead * d.W + kHead + 1;
-    chunk_sum_kernel<<<unsigned((n_part + 31) / 32), dim3(32, 8), 0, s>>>(
+    chunk_sum_kernel<<<unsigned((n_part + kSumValues - 1) / kSumValues), dim3(kSumValues, kSumLanes), 0, s>>>(
         at<float>(act, a.part), a.head_chunks, n_part, kHead * d.W, kHead, 1.0f / (4.0f * float(d.R)),
         grad + w_off(d, d.D), grad + b_off(d, d.D), loss_dev);
     RSI_CHECK_LAUNCH("chunk_sum_kernel");
@@ -634,7 +640,7 @@ extern "C" int rsi_nn_backward(const rsi_nn_net* net, const void* w16, const flo
         colsum_part_kernel<<<dim3(unsigned((d.W + 511) / 512), unsigned(chunks)), 256, 0, s>>>(
             dZ, d.R, d.W, at<float>(act, a.colpart));
         RSI_CHECK_LAUNCH("colsum_part_kernel");
-        chunk_sum_kernel<<<unsigned((d.W + 31) / 32), dim3(32, 8), 0, s>>>(
+        chunk_sum_kernel<<<unsigned(d.W / kSumValues), dim3(kSumValues, kSumLanes), 0, s>>>(
             at<float>(act, a.colpart), chunks, d.W, 0, d.W, 0.0f, nullptr, grad + b_off(d, l), nullptr);
         RSI_CHECK_LAUNCH("chunk_sum_kernel");
         if (l > 0) {
@@ -694,6 +700,11 @@ extern "C" int rsi_nn_infer(const rsi_nn_net* net, const void* w16, const float*
     const bool fused = net->engine == RSI_NN_ENGINE_TCGEN05 &&
                        ((reinterpret_cast<uintptr_t>(w16) | reinterpret_cast<uintptr_t>(w32)) & 15) == 0;
     const unsigned chunks = unsigned((d.npix + kChunk - 1) / kChunk);
+    for (int f0 = 0; f0 < n_fields; f0 += d.R) {  // (R fields' parameters fit p32)
+        rc = rsi_nn_carrier_coeffs(params + 5 * size_t(f0), std::min(d.R, n_fields - f0), net->c1, net->c2,
+                                   carrier + 4 * size_t(f0), at<float>(act, a.p32), stream);
+        if (rc != RSI_OK) return rc;
+    }
     for (int f0 = 0; f0 < n_fields; f0 += per) {
         const int nf = std::min(per, n_fields - f0);
         rc = rsi_nn_rows(net, params, n_fields, RSI_NN_ROWS_PIXELS, 0, nullptr, int64_t(f0) * d.npix, nullptr,
@@ -721,9 +732,6 @@ extern "C" int rsi_nn_infer(const rsi_nn_net* net, const void* w16, const float*
         }
         assemble_kernel<<<grid, 256, 0, s>>>(at<float4>(act, a.y), d.npix, chunk_sum, at<float2>(act, a.env));
         RSI_CHECK_LAUNCH("assemble_kernel");
-        rc = rsi_nn_carrier_coeffs(params + 5 * size_t(f0), nf, net->c1, net->c2, carrier + 4 * size_t(f0),
-                                   at<float>(act, a.p32), stream);
-        if (rc != RSI_OK) return rc;
         rc = rsi_nn_carrier(carrier + 4 * size_t(f0), nf, &net->window, +1, 1.0f, at<float>(act, a.env),
                             out + 2 * size_t(f0) * d.npix, stream);
         if (rc != RSI_OK) return rc;
