@@ -312,8 +312,8 @@ typedef struct rsi_raytrace {
     int32_t reserved;
 } rsi_raytrace;
 
-/* Workspace for rsi_raytrace_field (staged transducer tiles and split
- * partial sums); 0 on invalid input.                                      */
+/* Workspace for rsi_raytrace_field (staged transducer tiles, their clusters
+ * where the sum is offered them, split partial sums); 0 on invalid input.  */
 size_t rsi_raytrace_workspace_bytes(const rsi_raytrace *rt, int64_t n_src, int64_t n_tgt);
 
 /* Eq. transmitted_ray_tracing: for every target Q_j (in medium 2, z > z_I)
@@ -324,7 +324,9 @@ size_t rsi_raytrace_workspace_bytes(const rsi_raytrace *rt, int64_t n_src, int64
  * media; T12 of Eq. transmission_coefficient at the ray's angles).  Points
  * on the wrong side of the interface break the model: their sums come out
  * non-finite (recorded in the status word).  Same conventions for point
- * sets, field, workspace and stream as rsi_propagate_stage.                */
+ * sets, field, workspace and stream as rsi_propagate_stage.  With tile and
+ * newton 0, sums of 3e8 pairs and more may take far clusters of points through
+ * Chebyshev nodes, chosen on the device, as rsi_propagate_stage does.       */
 int rsi_raytrace_field(const rsi_raytrace *rt, const void *src_points, int64_t n_src,
                        const void *tgt_points, int64_t n_tgt, double *tgt_field,
                        void *workspace, size_t workspace_bytes, void *stream);

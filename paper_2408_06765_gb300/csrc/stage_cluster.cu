@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(kThreads, 4) leftover_kernel(const __grid_cons
     extern __shared__ __align__(128) uint8_t smem[];
     const auto& f = a.f[blockIdx.z];
     const int block = blockIdx.x / kTpt;
-    if (!gate_clustered(a.gate, a.S, a.gate_ratio) || !f.any[block]) return;
+    if (!f.any[block]) return;  // raised by the clustered kernel alone, so the gate need not be asked as well
     const Sum g = stage_sum(a, blockIdx.z);
     leftover_block<StageModel<KIND, NORM>, kTpt>(StageModel<KIND, NORM>{g}, g, block, blockIdx.x % kTpt, blockIdx.y,
                                                  a.segs, a.gate->L, a.gate->h,
