@@ -17,12 +17,6 @@
 // time-first list scheduling), so uneven instances balance across the SMs.
 // Each item writes its own partial-sum slot; the reduction adds the slots in
 // a fixed order, so results do not depend on the schedule.
-//
-// Stages long enough for the clustered kernel (stage_cluster.cu) leave the work
-// items and are captured as single stages on kBranches branches of the graph
-// beside the persistent kernel, each branch with a workspace of its own: a
-// scan of 64 instances of 2^12 .. 2^16 points and 128^2 pixels 38.7 -> 34.9 ms.
-// (Most of it are sums below that length: 2.8e8 pairs on average.)
 #include <string.h>
 
 #include <algorithm>
@@ -32,7 +26,6 @@
 
 #include "interface_body.cuh"
 #include "qmc_body.cuh"
-#include "stage.cuh"
 #include "stage_fp32_body.cuh"
 
 namespace {
@@ -103,7 +96,6 @@ struct BImage {
 };
 
 constexpr int kSeg = 256;
-constexpr int kBranches = 4;
 
 __global__ void batch_points_kernel(const BPointSet* __restrict__ sets, const BSeg* __restrict__ segs,
                                     rsi_qmc::SobolDirs dirs) {
@@ -256,8 +248,6 @@ struct rsi_batch_plan {
     uint64_t seed = 0;
     std::vector<size_t> o_pist, o_ifc, o_f1, o_sig, o_f2, o_t1, o_t2, o_p1, o_p2, img_off;
     std::vector<int> grid_id, S1, S2, tps1, tps2, sp1, sp2, nt1, nt2;
-    std::vector<bool> big1, big2;  // stages captured as single ones
-    size_t o_big = 0, big_bytes = 0;  // their workspaces: kBranches of big_bytes each
     std::vector<size_t> o_gridpts;
     std::vector<rsi_grid> grids;
     // captured graph
@@ -344,7 +334,7 @@ void build_tables(rsi_batch_plan& P, uint8_t* ws) {
             p.kind = RSI_STAGE_PISTON;
             p.normals = RSI_NORMALS_Z;
             prep1.push_back(p);
-            for (int t = 0; t < P.nt1[i] && !P.big1[i]; ++t) pt1.push_back({i, 0, t});
+            for (int t = 0; t < P.nt1[i]; ++t) pt1.push_back({i, 0, t});
             BStageInst s;
             s.tiles = p.tiles;
             s.tile_bytes = p.tile_bytes;
@@ -358,14 +348,14 @@ void build_tables(rsi_batch_plan& P, uint8_t* ws) {
             s.kl = float(I.k1 - double(s.kh));
             s.out = s.splits > 1 ? reinterpret_cast<double2*>(ws + P.o_p1[i]) : f1;
             st1.push_back(s);
-            int64_t blocks = P.big1[i] ? 0 : (I.n_iface + per_block - 1) / per_block;
+            int64_t blocks = (I.n_iface + per_block - 1) / per_block;
             for (int64_t b = 0; b < blocks; ++b)
                 for (int sp = 0; sp < s.splits; ++sp) {
                     int nt = std::min(s.n_tiles, (sp + 1) * s.tiles_per_split) - sp * s.tiles_per_split;
                     double cost = double(nt) * s.S * double(std::min<int64_t>(per_block, I.n_iface - b * per_block));
                     it1.push_back({cost, {i, sp, b}});
                 }
-            if (s.splits > 1 && !P.big1[i]) {
+            if (s.splits > 1) {
                 red1.push_back({s.out, f1, I.n_iface, s.splits, 0});
                 append_segments(rs1, int32_t(red1.size() - 1), I.n_iface);
             }
@@ -388,7 +378,7 @@ void build_tables(rsi_batch_plan& P, uint8_t* ws) {
             p.kind = RSI_STAGE_RSI;
             p.normals = P.normals2;
             prep2.push_back(p);
-            for (int t = 0; t < P.nt2[i] && !P.big2[i]; ++t) pt2.push_back({i, 0, t});
+            for (int t = 0; t < P.nt2[i]; ++t) pt2.push_back({i, 0, t});
             BStageInst s;
             s.tiles = p.tiles;
             s.tile_bytes = p.tile_bytes;
@@ -402,14 +392,14 @@ void build_tables(rsi_batch_plan& P, uint8_t* ws) {
             s.kl = float(I.k2 - double(s.kh));
             s.out = s.splits > 1 ? reinterpret_cast<double2*>(ws + P.o_p2[i]) : f2;
             st2.push_back(s);
-            int64_t blocks = P.big2[i] ? 0 : (n_g + per_block - 1) / per_block;
+            int64_t blocks = (n_g + per_block - 1) / per_block;
             for (int64_t b = 0; b < blocks; ++b)
                 for (int sp = 0; sp < s.splits; ++sp) {
                     int nt = std::min(s.n_tiles, (sp + 1) * s.tiles_per_split) - sp * s.tiles_per_split;
                     double cost = double(nt) * s.S * double(std::min<int64_t>(per_block, n_g - b * per_block));
                     it2.push_back({cost, {i, sp, b}});
                 }
-            if (s.splits > 1 && !P.big2[i]) {
+            if (s.splits > 1) {
                 red2.push_back({s.out, f2, n_g, s.splits, 0});
                 append_segments(rs2, int32_t(red2.size() - 1), n_g);
             }
@@ -510,87 +500,8 @@ int launch_batch_stage_v(const rsi_batch_plan& P, uint8_t* ws, size_t o_st, size
     return launch_batch_stage<KIND, NORM, 2, 2>(P, ws, o_st, o_it, n_items, max_tile, ctr, status, s);
 }
 
-rsi_stage batch_stage(const rsi_batch_instance& I, bool second) {
-    rsi_stage st = {};
-    st.kind = second ? RSI_STAGE_RSI : RSI_STAGE_PISTON;
-    st.precision = RSI_PREC_FP32C;
-    st.k = second ? I.k2 : I.k1;
-    st.v0 = second ? 1.0 : I.v0;
-    st.normals = RSI_NORMALS_Z;
-    return st;
-}
-
-// The branches of the graph that the single stages are captured on
-struct Branches {
-    cudaStream_t s[kBranches] = {};
-    cudaEvent_t fork = nullptr, join[kBranches] = {};
-    int create() {
-        RSI_CUDA_TRY(cudaEventCreateWithFlags(&fork, cudaEventDisableTiming), "cudaEventCreate");
-        for (int b = 0; b < kBranches; ++b) {
-            RSI_CUDA_TRY(cudaStreamCreateWithFlags(&s[b], cudaStreamNonBlocking), "cudaStreamCreate");
-            RSI_CUDA_TRY(cudaEventCreateWithFlags(&join[b], cudaEventDisableTiming), "cudaEventCreate");
-        }
-        return RSI_OK;
-    }
-    ~Branches() {
-        for (int b = 0; b < kBranches; ++b) {
-            if (join[b]) cudaEventDestroy(join[b]);
-            if (s[b]) cudaStreamDestroy(s[b]);
-        }
-        if (fork) cudaEventDestroy(fork);
-    }
-};
-
-// Fork the branches off `s` and put the single stages on them, the longest first
-// and each to the branch with the fewest pairs so far; join() waits for them.
-int fork_stages(rsi_batch_plan& P, uint8_t* ws, bool second, Branches& br, int* status, cudaStream_t s) {
-    const std::vector<bool>& big = second ? P.big2 : P.big1;
-    std::vector<std::pair<double, int>> order;
-    for (int i = 0; i < P.n_inst; ++i)
-        if (big[i])
-            order.push_back({double(P.inst[i].n_iface) * double(second ? int64_t(P.grids[P.grid_id[i]].nx) *
-                                                                             P.grids[P.grid_id[i]].nz
-                                                                       : P.inst[i].n_piston),
-                             i});
-    if (order.empty()) return RSI_OK;
-    std::stable_sort(order.begin(), order.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
-    RSI_CUDA_TRY(cudaEventRecord(br.fork, s), "cudaEventRecord");
-    for (int b = 0; b < kBranches; ++b) RSI_CUDA_TRY(cudaStreamWaitEvent(br.s[b], br.fork, 0), "cudaStreamWaitEvent");
-    double load[kBranches] = {};
-    for (auto& e : order) {
-        const int i = e.second, b = int(std::min_element(load, load + kBranches) - load);
-        load[b] += e.first;
-        const rsi_batch_instance& I = P.inst[i];
-        const PointsView ifc = rsi_points_view(ws + P.o_ifc[i], I.n_iface);
-        const rsi_stage st = batch_stage(I, second);
-        uint8_t* work = ws + P.o_big + size_t(b) * P.big_bytes;
-        int rc;
-        if (second) {
-            const rsi_grid& g = P.grids[P.grid_id[i]];
-            const int64_t n_g = int64_t(g.nx) * g.nz;
-            rc = stage_clustered_run(st, ifc, I.n_iface, reinterpret_cast<const double2*>(ws + P.o_sig[i]),
-                                     rsi_points_view(ws + P.o_gridpts[P.grid_id[i]], n_g), n_g,
-                                     reinterpret_cast<double2*>(ws + P.o_f2[i]), work, status, br.s[b]);
-        } else {
-            rc = stage_clustered_run(st, rsi_points_view(ws + P.o_pist[i], I.n_piston), I.n_piston, nullptr, ifc,
-                                     I.n_iface, reinterpret_cast<double2*>(ws + P.o_f1[i]), work, status, br.s[b]);
-        }
-        if (rc != RSI_OK) return rc;
-    }
-    return RSI_OK;
-}
-int join_stages(rsi_batch_plan& P, bool second, Branches& br, cudaStream_t s) {
-    const std::vector<bool>& big = second ? P.big2 : P.big1;
-    if (std::find(big.begin(), big.end(), true) == big.end()) return RSI_OK;
-    for (int b = 0; b < kBranches; ++b) {
-        RSI_CUDA_TRY(cudaEventRecord(br.join[b], br.s[b]), "cudaEventRecord");
-        RSI_CUDA_TRY(cudaStreamWaitEvent(s, br.join[b], 0), "cudaStreamWaitEvent");
-    }
-    return RSI_OK;
-}
-
 // Enqueue the whole batch on `s` (captured into the graph by rsi_batch_run).
-int enqueue(rsi_batch_plan& P, uint8_t* ws, Branches& br, int* status, cudaStream_t s) {
+int enqueue(rsi_batch_plan& P, uint8_t* ws, int* status, cudaStream_t s) {
     static const rsi_qmc::SobolDirs dirs = rsi_qmc::make_dirs();
     unsigned long long* ctr = reinterpret_cast<unsigned long long*>(ws + P.o_ctr);
     RSI_CUDA_TRY(cudaMemsetAsync(ctr, 0, 2 * sizeof(unsigned long long), s), "reset work counters");
@@ -604,49 +515,37 @@ int enqueue(rsi_batch_plan& P, uint8_t* ws, Branches& br, int* status, cudaStrea
                                                                reinterpret_cast<const BSeg*>(ws + P.o_gsegs));
         RSI_CHECK_LAUNCH("batch_grid_kernel");
     }
-    int rc = fork_stages(P, ws, false, br, status, s);
+    batch_prep_kernel<<<unsigned(P.n_pt1), P.S_max, 0, s>>>(reinterpret_cast<const BPrep*>(ws + P.o_prep1),
+                                                            reinterpret_cast<const BPrepTile*>(ws + P.o_pt1),
+                                                            P.variant == 3 ? 1 : 0);
+    RSI_CHECK_LAUNCH("batch_prep_kernel");
+    int rc = launch_batch_stage_v<RSI_STAGE_PISTON, RSI_NORMALS_Z>(P, ws, P.o_st1, P.o_it1, P.n_it1, P.max_tile1,
+                                                                   ctr, status, s);
     if (rc != RSI_OK) return rc;
-    if (P.n_pt1) {
-        batch_prep_kernel<<<unsigned(P.n_pt1), P.S_max, 0, s>>>(reinterpret_cast<const BPrep*>(ws + P.o_prep1),
-                                                                reinterpret_cast<const BPrepTile*>(ws + P.o_pt1),
-                                                                P.variant == 3 ? 1 : 0);
-        RSI_CHECK_LAUNCH("batch_prep_kernel");
-        rc = launch_batch_stage_v<RSI_STAGE_PISTON, RSI_NORMALS_Z>(P, ws, P.o_st1, P.o_it1, P.n_it1, P.max_tile1, ctr,
-                                                                   status, s);
-        if (rc != RSI_OK) return rc;
-    }
     if (P.n_rs1) {
         batch_reduce_kernel<<<unsigned(P.n_rs1), kSeg, 0, s>>>(reinterpret_cast<const BReduce*>(ws + P.o_red1),
                                                                reinterpret_cast<const BSeg*>(ws + P.o_rs1), status);
         RSI_CHECK_LAUNCH("batch_reduce_kernel");
     }
-    rc = join_stages(P, false, br, s);
-    if (rc != RSI_OK) return rc;
     batch_transmit_kernel<<<unsigned(P.n_ts), kSeg, 0, s>>>(reinterpret_cast<const BTransmit*>(ws + P.o_tr),
                                                             reinterpret_cast<const BSeg*>(ws + P.o_ts));
     RSI_CHECK_LAUNCH("batch_transmit_kernel");
-    rc = fork_stages(P, ws, true, br, status, s);
+    batch_prep_kernel<<<unsigned(P.n_pt2), P.S_max, 0, s>>>(reinterpret_cast<const BPrep*>(ws + P.o_prep2),
+                                                            reinterpret_cast<const BPrepTile*>(ws + P.o_pt2),
+                                                            P.variant == 3 ? 1 : 0);
+    RSI_CHECK_LAUNCH("batch_prep_kernel");
+    if (P.normals2 == RSI_NORMALS_POINTS)
+        rc = launch_batch_stage_v<RSI_STAGE_RSI, RSI_NORMALS_POINTS>(P, ws, P.o_st2, P.o_it2, P.n_it2, P.max_tile2,
+                                                                     ctr + 1, status, s);
+    else
+        rc = launch_batch_stage_v<RSI_STAGE_RSI, RSI_NORMALS_Z>(P, ws, P.o_st2, P.o_it2, P.n_it2, P.max_tile2,
+                                                                ctr + 1, status, s);
     if (rc != RSI_OK) return rc;
-    if (P.n_pt2) {
-        batch_prep_kernel<<<unsigned(P.n_pt2), P.S_max, 0, s>>>(reinterpret_cast<const BPrep*>(ws + P.o_prep2),
-                                                                reinterpret_cast<const BPrepTile*>(ws + P.o_pt2),
-                                                                P.variant == 3 ? 1 : 0);
-        RSI_CHECK_LAUNCH("batch_prep_kernel");
-        if (P.normals2 == RSI_NORMALS_POINTS)
-            rc = launch_batch_stage_v<RSI_STAGE_RSI, RSI_NORMALS_POINTS>(P, ws, P.o_st2, P.o_it2, P.n_it2, P.max_tile2,
-                                                                         ctr + 1, status, s);
-        else
-            rc = launch_batch_stage_v<RSI_STAGE_RSI, RSI_NORMALS_Z>(P, ws, P.o_st2, P.o_it2, P.n_it2, P.max_tile2,
-                                                                    ctr + 1, status, s);
-        if (rc != RSI_OK) return rc;
-    }
     if (P.n_rs2) {
         batch_reduce_kernel<<<unsigned(P.n_rs2), kSeg, 0, s>>>(reinterpret_cast<const BReduce*>(ws + P.o_red2),
                                                                reinterpret_cast<const BSeg*>(ws + P.o_rs2), status);
         RSI_CHECK_LAUNCH("batch_reduce_kernel");
     }
-    rc = join_stages(P, true, br, s);
-    if (rc != RSI_OK) return rc;
     batch_image_kernel<<<unsigned(P.n_is), kSeg, 0, s>>>(reinterpret_cast<const BImage*>(ws + P.o_imgtab),
                                                          reinterpret_cast<const BSeg*>(ws + P.o_is));
     RSI_CHECK_LAUNCH("batch_image_kernel");
@@ -739,14 +638,6 @@ extern "C" int rsi_batch_create(const rsi_batch_instance* inst, int32_t n_inst, 
         P->tps2.push_back(tps2);
         P->sp1.push_back(sp1);
         P->sp2.push_back(sp2);
-        // an automatic shape only: a given one keeps the persistent kernel's
-        const bool automatic = !shape || (!shape->tile && !shape->tpt && !shape->variant);
-        const size_t big1 = automatic ? stage_clustered_bytes(batch_stage(I, false), I.n_piston, I.n_iface) : 0;
-        const size_t big2 = automatic && P->normals2 == RSI_NORMALS_Z
-                                ? stage_clustered_bytes(batch_stage(I, true), I.n_iface, n_g) : 0;
-        P->big1.push_back(big1 > 0);
-        P->big2.push_back(big2 > 0);
-        P->big_bytes = std::max(P->big_bytes, align256(std::max(big1, big2)));
         size_t tb1 = RSI_TILE_HDR_BYTES + size_t(S1) * 32, tb2 = RSI_TILE_HDR_BYTES + size_t(S2) * rec2;
         P->max_tile1 = std::max(P->max_tile1, tb1);
         P->max_tile2 = std::max(P->max_tile2, tb2);
@@ -755,14 +646,13 @@ extern "C" int rsi_batch_create(const rsi_batch_instance* inst, int32_t n_inst, 
         P->o_f1.push_back(take(size_t(I.n_iface) * 16));
         P->o_sig.push_back(take(size_t(I.n_iface) * 16));
         P->o_f2.push_back(take(size_t(n_g) * 16));
-        P->o_t1.push_back(take(big1 ? 0 : size_t(nt1) * tb1));
-        P->o_t2.push_back(take(big2 ? 0 : size_t(nt2) * tb2));
-        P->o_p1.push_back(sp1 > 1 && !big1 ? take(size_t(sp1) * size_t(I.n_iface) * 16) : 0);
-        P->o_p2.push_back(sp2 > 1 && !big2 ? take(size_t(sp2) * size_t(n_g) * 16) : 0);
+        P->o_t1.push_back(take(size_t(nt1) * tb1));
+        P->o_t2.push_back(take(size_t(nt2) * tb2));
+        P->o_p1.push_back(sp1 > 1 ? take(size_t(sp1) * size_t(I.n_iface) * 16) : 0);
+        P->o_p2.push_back(sp2 > 1 ? take(size_t(sp2) * size_t(n_g) * 16) : 0);
         P->img_off.push_back(P->img_elems);
         P->img_elems += size_t(n_g);
     }
-    P->o_big = take(size_t(kBranches) * P->big_bytes);
     const size_t buffers = align256(off);
     // tables: build once against base 0 to learn their size, then shift every
     // buffer offset past them
@@ -779,7 +669,6 @@ extern "C" int rsi_batch_create(const rsi_batch_instance* inst, int32_t n_inst, 
     shift(P->o_f2);
     shift(P->o_t1);
     shift(P->o_t2);
-    P->o_big += tables;
     for (int i = 0; i < n_inst; ++i) {
         if (P->sp1[i] > 1) P->o_p1[i] += tables;
         if (P->sp2[i] > 1) P->o_p2[i] += tables;
@@ -816,21 +705,13 @@ extern "C" int rsi_batch_run(rsi_batch_plan* P, void* workspace, size_t workspac
         // capture the whole batch once; later runs replay the graph
         cudaStream_t cap = nullptr;
         RSI_CUDA_TRY(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking), "cudaStreamCreate");
-        Branches br;
-        {
-            const int brc = br.create();
-            if (brc != RSI_OK) {
-                cudaStreamDestroy(cap);
-                return brc;
-            }
-        }
         cudaGraph_t graph = nullptr;
         cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) {
             cudaStreamDestroy(cap);
             return rsi_cuda_fail(e, "cudaStreamBeginCapture");
         }
-        int rc = enqueue(*P, ws, br, status, cap);
+        int rc = enqueue(*P, ws, status, cap);
         e = cudaStreamEndCapture(cap, &graph);
         cudaStreamDestroy(cap);
         if (rc != RSI_OK) {

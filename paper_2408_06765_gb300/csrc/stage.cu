@@ -209,56 +209,6 @@ int make_plan(const rsi_stage& st, int64_t n_src, int64_t n_tgt, Plan& p, int ma
     return RSI_OK;
 }
 
-// The launches of a planned stage; `timed`: between the events of rsi_timing
-// (which a captured stage must not record).
-int run_plan(const rsi_stage& st, const Plan& p, const PointsView& src, int64_t n_src, const double2* sigma,
-             const PointsView& tgt, int64_t n_tgt, double2* field, uint8_t* tiles, int* status, bool timed,
-             cudaStream_t s) {
-    const bool fp32 = st.precision == RSI_PREC_FP32C;
-    StageArgs a = {};
-    a.kind = st.kind;
-    a.normals = st.kind == RSI_STAGE_RSI ? base_normals(st.normals) : RSI_NORMALS_Z;
-    a.tpt = p.tpt;
-    a.variant = p.variant;
-    a.S = p.S;
-    a.n_tiles = p.n_tiles;
-    a.tiles_per_split = p.tiles_per_split;
-    a.splits = p.splits;
-    a.n_tgt = n_tgt;
-    a.tile_bytes = p.tile_bytes;
-    a.tiles = tiles;
-    a.tgt = {tgt.xh, tgt.xl, tgt.yh, tgt.yl, tgt.zh, tgt.zl, tgt.x, tgt.y, tgt.z};
-    a.k = st.k;
-    a.kh = float(st.k);
-    a.kl = float(st.k - double(a.kh));
-    a.tp = two_pi_split();
-    a.out = p.splits > 1 ? reinterpret_cast<double2*>(tiles + p.part_at()) : field;
-    a.status = status;
-    TimingScope tsc;
-    if (p.clustered) {
-        ClusterArgs c;
-        int rc = cluster_prepare(st, &st.k, 1.0f, src, n_src, sigma, a.tgt, n_tgt, field, p.c, tiles, status, c, s);
-        if (rc != RSI_OK) return rc;
-        a.gate = c.gate;
-        a.gate_ratio = c.gate_ratio;
-        if (timed) tsc = timing_begin(s);
-        rc = cluster_run(c, s);
-        if (rc == RSI_OK) rc = launch_stage_fp32(a, s);
-        if (rc != RSI_OK) return rc;
-        if (timed) timing_end(tsc, st.kind, double(n_src) * double(n_tgt), s);
-        return p.splits > 1 ? launch_reduce_gated(a, field, s) : RSI_OK;
-    }
-    int rc = fp32 ? launch_prep_fp32(st, src, n_src, sigma, p.S, tiles, p.tile_bytes, p.n_tiles, s, p.variant == 3)
-                  : launch_prep_fp64(st, src, n_src, sigma, p.S, tiles, p.tile_bytes, p.n_tiles, s);
-    if (rc != RSI_OK) return rc;
-    if (timed) tsc = timing_begin(s);
-    rc = fp32 ? launch_stage_fp32(a, s) : launch_stage_fp64(a, s);
-    if (rc != RSI_OK) return rc;
-    if (timed) timing_end(tsc, st.kind, double(n_src) * double(n_tgt), s);
-    if (p.splits > 1) return launch_reduce_partials(a.out, p.splits, n_tgt, field, status, s);
-    return RSI_OK;
-}
-
 }  // namespace
 
 extern "C" size_t rsi_stage_workspace_bytes(const rsi_stage* st, int64_t n_src, int64_t n_tgt) {
@@ -298,22 +248,54 @@ extern "C" int rsi_propagate_stage(const rsi_stage* st, const void* src_points, 
         return rsi_fail(RSI_E_NOMEM, "rsi_propagate_stage: workspace %zu < %zu bytes", workspace_bytes, p.bytes());
     int* status = rsi_status_ptr();
     if (!status) return RSI_E_CUDA;
-    return run_plan(*st, p, rsi_points_view(const_cast<void*>(src_points), n_src), n_src,
-                    reinterpret_cast<const double2*>(src_sigma), rsi_points_view(const_cast<void*>(tgt_points), n_tgt),
-                    n_tgt, reinterpret_cast<double2*>(tgt_field), static_cast<uint8_t*>(workspace), status, true,
-                    static_cast<cudaStream_t>(stream));
-}
-
-size_t stage_clustered_bytes(const rsi_stage& st, int64_t n_src, int64_t n_tgt) {
-    Plan p;
-    return make_plan(st, n_src, n_tgt, p) == RSI_OK && p.clustered ? p.bytes() : 0;
-}
-int stage_clustered_run(const rsi_stage& st, const PointsView& src, int64_t n_src, const double2* sigma,
-                        const PointsView& tgt, int64_t n_tgt, double2* field, uint8_t* workspace, int* status,
-                        cudaStream_t s) {
-    Plan p;
-    const int rc = make_plan(st, n_src, n_tgt, p);
-    return rc != RSI_OK ? rc : run_plan(st, p, src, n_src, sigma, tgt, n_tgt, field, workspace, status, false, s);
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    const bool fp32 = st->precision == RSI_PREC_FP32C;
+    PointsView src = rsi_points_view(const_cast<void*>(src_points), n_src);
+    PointsView tgt = rsi_points_view(const_cast<void*>(tgt_points), n_tgt);
+    uint8_t* tiles = static_cast<uint8_t*>(workspace);
+    const double2* sigma = reinterpret_cast<const double2*>(src_sigma);
+    StageArgs a = {};
+    a.kind = st->kind;
+    a.normals = st->kind == RSI_STAGE_RSI ? base_normals(st->normals) : RSI_NORMALS_Z;
+    a.tpt = p.tpt;
+    a.variant = p.variant;
+    a.S = p.S;
+    a.n_tiles = p.n_tiles;
+    a.tiles_per_split = p.tiles_per_split;
+    a.splits = p.splits;
+    a.n_tgt = n_tgt;
+    a.tile_bytes = p.tile_bytes;
+    a.tiles = tiles;
+    a.tgt = {tgt.xh, tgt.xl, tgt.yh, tgt.yl, tgt.zh, tgt.zl, tgt.x, tgt.y, tgt.z};
+    a.k = st->k;
+    a.kh = float(st->k);
+    a.kl = float(st->k - double(a.kh));
+    a.tp = two_pi_split();
+    double2* field = reinterpret_cast<double2*>(tgt_field);
+    a.out = p.splits > 1 ? reinterpret_cast<double2*>(tiles + p.part_at()) : field;
+    a.status = status;
+    if (p.clustered) {
+        ClusterArgs c;
+        rc = cluster_prepare(*st, &st->k, 1.0f, src, n_src, sigma, a.tgt, n_tgt, field, p.c, tiles, status, c, s);
+        if (rc != RSI_OK) return rc;
+        a.gate = c.gate;
+        a.gate_ratio = c.gate_ratio;
+        TimingScope tsc = timing_begin(s);
+        rc = cluster_run(c, s);
+        if (rc == RSI_OK) rc = launch_stage_fp32(a, s);
+        if (rc != RSI_OK) return rc;
+        timing_end(tsc, st->kind, double(n_src) * double(n_tgt), s);
+        return p.splits > 1 ? launch_reduce_gated(a, field, s) : RSI_OK;
+    }
+    rc = fp32 ? launch_prep_fp32(*st, src, n_src, sigma, p.S, tiles, p.tile_bytes, p.n_tiles, s, p.variant == 3)
+              : launch_prep_fp64(*st, src, n_src, sigma, p.S, tiles, p.tile_bytes, p.n_tiles, s);
+    if (rc != RSI_OK) return rc;
+    TimingScope tsc = timing_begin(s);
+    rc = fp32 ? launch_stage_fp32(a, s) : launch_stage_fp64(a, s);
+    if (rc != RSI_OK) return rc;
+    timing_end(tsc, st->kind, double(n_src) * double(n_tgt), s);
+    if (p.splits > 1) return launch_reduce_partials(a.out, p.splits, n_tgt, field, status, s);
+    return RSI_OK;
 }
 
 TimingScope timing_begin(cudaStream_t s) {

@@ -91,14 +91,6 @@ struct StageArgs {
     float gate_ratio;
 };
 
-// For callers that capture many stages (batch.cu): the workspace of a stage that
-// is offered the clustered kernel (0: it is not), and its launches, untimed, for
-// an automatic shape; the workspace is 256-byte aligned.
-size_t stage_clustered_bytes(const rsi_stage& st, int64_t n_src, int64_t n_tgt);
-int stage_clustered_run(const rsi_stage& st, const PointsView& src, int64_t n_src, const double2* sigma,
-                        const PointsView& tgt, int64_t n_tgt, double2* field, uint8_t* workspace, int* status,
-                        cudaStream_t s);
-
 size_t fp32_record_bytes(int kind, int normals);
 double stage_amp_scale(const rsi_stage& st);  // -v0/(2 pi) (piston) or -+1/(2 pi) (RSI)
 // Reversed normals (RSI_NORMALS_NEG_Z, RSI_NORMALS_POINTS_NEG): cos(theta) is
@@ -185,3 +177,4 @@ void timing_end(TimingScope& t, int kind, double pairs, cudaStream_t s);
 int launch_reduce_partials(const double2* part, int splits, int64_t n, double2* out, int* status, cudaStream_t s);
 // the same for the direct kernel beside the clustered one: nothing is done where the gate chose the other
 int launch_reduce_gated(const StageArgs& a, double2* out, cudaStream_t s);
+

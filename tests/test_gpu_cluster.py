@@ -133,28 +133,3 @@ def test_raytrace_matches_direct_and_oracle(case):
     want = torch.from_numpy(oracle.raytrace_image(cfg, pixels=px))
     got, ref = (v.reshape(-1).cpu()[torch.from_numpy(px)] for v in (clustered, direct))
     assert rel(got, want) <= rel(ref, want) + TOL
-
-
-def test_batch_captures_long_stages_beside_the_others():
-    """Instances whose piston stage, both stages or neither are long enough for
-    the clustered kernel, in one graph, against the same chains one by one; run
-    twice, and an explicit shape (the persistent kernel alone)."""
-    counts = np.zeros((workloads.C4_NFREQ * workloads.C4_NPOS, 2), np.int64)
-    pick = {(3, 1): (9001, 60001), (40, 5): (4096, 5003), (20, 2): (8192, 65536), (61, 9): (65536, 8209)}
-    for (jf, pos), n in pick.items():
-        counts[jf * workloads.C4_NPOS + pos] = n
-    cfgs = [workloads.c4_instance(jf, pos, counts) for jf, pos in pick]
-    for i, c in enumerate(cfgs):
-        c["grid"].update({"nx": 131, "nz": 129})
-        c["piston"]["set_id"], c["interfaces"][0]["set_id"] = 2 * i, 2 * i + 1
-    batch = rsi.Batch(cfgs, seed=1)
-    first = batch.run().clone()
-    assert torch.equal(batch.run(), first)
-    shaped = rsi.Batch(cfgs, seed=1, shape=rsi.stage_struct(rsi.STAGE_RSI, "fp32c", 1.0, tile=256))
-    direct = shaped.run()
-    assert not torch.equal(first, direct) and rel(first, direct) <= TOL
-    for i, c in enumerate(cfgs):
-        assert rel(batch.image(i), rsi.run_chain(dict(c, seed=1), fmt="c64").image) <= TOL
-    rsi.sync_status()
-    batch.close()
-    shaped.close()
