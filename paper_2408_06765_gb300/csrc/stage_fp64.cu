@@ -4,9 +4,9 @@
 // phase and 48-bit amplitudes (stage_fp64_body.cuh), summed in pairs of floats
 // over 32 terms and in doubles with Neumaier compensation over those.
 // 2^12 x 2^12 pairs of a piston stage: 2.08 ms with every operation in doubles
-// (75 of the FP64 pipe per pair, 98 % of the time), 0.50 ms now, of which the
-// pipe's 12 operations take 0.35; of an interface stage 2.37 and 0.50 (0.60 with
-// per-point normals, 15 operations).
+// (54 double instructions per pair), 0.40 ms now with 9.7, 0.92 of what the
+// pipe's rate allows for them; of an interface stage 2.37 and 0.40 (per-point
+// normals, 3 operations more: 2.46 and 0.49).
 #include <math.h>
 
 #include "stage_fp64_body.cuh"

@@ -2,14 +2,15 @@
 //
 // The chip's FP64 pipe takes 2 lanes per cycle and SM, 1/64 of the FP32 and
 // integer rate, and the term spelled out in doubles (square root, division,
-// sincos, compensated sums) is 75 operations of that pipe: 7.6 Gpair/s, all of
-// it pipe time.  Only what decides the phase needs 53 bits, since a path is
-// hundreds of radians long: the offset, its square, the first estimate g of
-// the distance and k g less whole turns, 12 operations.  From there on the
+// sincos, compensated sums) is 54 double instructions (63 for an interface) and
+// comparisons of that pipe, which they kept busy: 8 Gpair/s.  Only what decides
+// the phase needs 53 bits, since a path is hundreds of radians long: the offset,
+// its square, the first estimate g of the distance, its error and k g less whole
+// turns, 9 operations.  From there on the
 // numbers are of the order of one and go on as integers (the phase, in units of
 // 2^-50 quarter turns) and as pairs of floats of 48 bits (sine and cosine from a
 // table, amplitude, products, runs of 32 terms): some 150 FP32 and integer
-// operations beside the 12, which leave the FP64 pipe the bound.  The error of a
+// operations beside the 9, which leave the FP64 pipe the bound.  The error of a
 // term stays with the rounding of the squared distance, as in doubles
 // throughout; the phase itself is no longer rounded at the size of k r.
 #pragma once
@@ -41,6 +42,11 @@ __device__ __forceinline__ DF df_add(const DF& a, const DF& b) {
 }
 __device__ __forceinline__ DF df_neg(const DF& a) { return {-a.h, -a.l}; }
 
+// a float as a double by moving bits; normal or 0
+__device__ __forceinline__ double widen(float f) {
+    const int b = __float_as_int(f);
+    return b << 1 ? __hiloint2double(((b & 0x7fffffff) >> 3) + 0x38000000 | (b & 0x80000000), b << 29) : 0.0;
+}
 // A double as a pair of floats by moving bits (a conversion would be FP64 pipe
 // time): the leading 24 bits of the significand, truncated, and the other 29.
 // |d| < 2^127; below 2^-74: 0.
@@ -96,7 +102,7 @@ constexpr Tab make_tab() {
 // k and what is made of it once per thread
 struct Wave {
     double k, kq;        // kq = 2 k / pi: quarter turns per metre
-    float rho;           // (2 k / pi - kq) / kq
+    float kqf, rho;      // kq in single precision; (2 k / pi - kq) / kq
     DF kf;
     unsigned first, span;  // high words of the squared distances that fast_term takes
 };
@@ -105,6 +111,7 @@ __device__ __forceinline__ Wave make_wave(double k) {
     w.k = k;
     const double ch = 0.63661977236758138, cl = -3.9357353350364972e-17;  // 2 / pi
     w.kq = k * ch;
+    w.kqf = float(w.kq);
     w.rho = float((fma(k, ch, -w.kq) + k * cl) / w.kq);
     w.kf.h = float(k);
     w.kf.l = float(k - double(w.kf.h));
@@ -123,20 +130,20 @@ __device__ __forceinline__ bool in_range(const Wave& w, double r2) {
 // 1/r and e^{ikr} for a squared distance in range
 __device__ __forceinline__ void fast_wave(const Wave& w, double r2, const TabEntry* __restrict__ tab, DF& ir, DF& c,
                                           DF& s) {
-    const float y0 = rsqrt_approx(leading_float(__double2hiint(r2), __double2loint(r2)));
-    const int yb = __float_as_int(y0);
-    const double y = __hiloint2double((yb >> 3) + 0x38000000, yb << 29);
+    const float rf = leading_float(__double2hiint(r2), __double2loint(r2));
+    const float y0 = rsqrt_approx(rf);
+    const double y = widen(y0);
     // r = g (1 - u)^(-1/2), 1 - u = g y, |u| < 2^-21: 2.5 - g y lies in [1, 2),
     // so the low word of the sum is u in units of 2^-52
     const double g = r2 * y;
     const int ui = __double2loint(__fma_rn(-g, y, 2.5));
-    const double magic = 6755399441055744.0;  // 1.5 2^52
-    const double m = __fma_rn(g, w.kq, magic);
-    const double f = __fma_rn(g, w.kq, __dsub_rn(magic, m));  // quarter turns less whole ones, [-1/2, 1/2]
-    const int n = __double2loint(m);
-    long long x = __double_as_longlong(__dadd_rn(f, 6.0)) - 0x4018000000000000ll;  // units of 2^-50
+    // whole quarter turns n by single precision: off by 0.1 at most, so f = kq g - n
+    // stays within 0.6 and 6 + f in [4, 8), where a double's last bit is 2^-50
+    const float nf = rintf(__fmul_rn(__fmul_rn(rf, y0), w.kqf));
+    const int n = int(nf);
+    long long x = __double_as_longlong(__fma_rn(g, w.kq, widen(__fsub_rn(6.0f, nf)))) - 0x4018000000000000ll;
     // r - g and the rest of kq: kq (r - g) = (n + f)(u/2 + 3 u^2/8), n rho
-    const float nf = float(n), ff = __fmul_rn(float(int(x >> 21)), 0x1p-29f);
+    const float ff = __fmul_rn(float(int(x >> 21)), 0x1p-29f);
     const float hu = __fmul_rn(float(ui >> 8), 0x1p-45f), hul = __fmul_rn(float(ui & 255), 0x1p-53f);  // u / 2
     const float u2 = __fmaf_rn(__fmul_rn(1.5f, hu), hu, hul);  // 3 u^2 / 8 and the low part of u / 2
     const float p = __fmul_rn(nf, hu);
