@@ -226,6 +226,12 @@ bool cluster_plan(int kind, int normals, int nf, int64_t n_src, int64_t n_tgt, i
     p.splits = int((roots + rps - 1) / rps);
     p.top = top(rps);
     p.fill = float(std::min(1.0, double(blocks * p.splits * nf) / double(slots)));
+    // With few blocks of targets a CTA's own time and the preparation decide, which
+    // the estimate does not see.  Direct and clustered, ms: rays from 44069 points
+    // onto 8 blocks 2.07, 3.01; piston 65536 onto 9 0.50, 0.54, 30000 onto 24 0.60,
+    // 0.64; interface 120000 onto 9 0.90, 1.01, but 262144 onto 5, 64 roots for
+    // their CTAs, 1.04, 0.76 and 65536 onto 16 0.88, 0.75; rays from 16384 onto 32 2.32, 1.77
+    if (blocks < (kind == RSI_STAGE_PISTON ? 32 : 16) && roots < 64) return false;
     // what the 60 us of launches and CTAs' set-up, at 9.2e11 instructions per warp
     // and second, leave of the direct sum's time for the clusters' arithmetic
     // (134.4 instructions per source and 256 targets)
@@ -238,9 +244,10 @@ bool cluster_plan(int kind, int normals, int nf, int64_t n_src, int64_t n_tgt, i
     p.any_at = p.left_at + align256(size_t(nf) * size_t(blocks) * size_t(n_tiles));
     p.extra_bytes = p.any_at + align256(size_t(nf) * size_t(blocks) * sizeof(int)) + 256;
     // 16 segments: a block next to the sources is left whole, and its four
-    // quarters are then 64 CTAs' work; fewer where the sum has blocks enough
-    // (at most 2^24 partial sums)
-    p.segs = int(std::max<int64_t>(1, std::min<int64_t>({16, n_tiles / 4, (int64_t(1) << 24) / n_tgt})));
+    // quarters are then 64 CTAs' work; more where there are few blocks, fewer where
+    // there are many (at most 2^24 partial sums)
+    p.segs = int(std::max<int64_t>(1, std::min<int64_t>({std::max<int64_t>(16, 608 / blocks), n_tiles / 4,
+                                                         (int64_t(1) << 24) / n_tgt})));
     p.partial_bytes = align256(size_t(p.splits + p.segs) * size_t(n_tgt) * sizeof(double2));
     return true;
 }
