@@ -76,7 +76,7 @@ struct alignas(16) WarpArea {
     float2 y[kMaxNN];        // between the two passes of a transform
     float2 fh[kMaxNN];       // Chebyshev coefficients of the field on the target cluster
     Node node;
-    float D1h, D1l, D2h, D2l, S0h, S0l;  // block centre - cluster centre along the block's axes, its square
+    float D1h, D1l, D2h, D2l, S0h, S0l;  // prepare_targets' D along the block's axes, and |D|^2
     int item;                // level, tile, target cluster, N (0: none)
     int pad;
 };
@@ -587,13 +587,17 @@ struct StageModel {
         const float2 x = __ffma2_rn(__fadd2_rn(__ffma2_rn(ph, dup(0.5f), magic), nmagic), dup(-2.0f), ph);
         return __fadd2_rn(x, __fadd2_rn(pl, dup(r.tau)));
     }
-    // for the targets' phases: the block's centre from the cluster's, exactly (one lane)
+    // for the targets' phases (one lane): D from the cluster's centre, exactly, to
+    // the block's centre along the rectangles' axes, from which run_block counts
+    // the targets' offsets, and to the rectangle's own plane across them: where a
+    // block spans several planes, a quarter of it may lie in one
     __device__ __forceinline__ void prepare_targets(WarpArea& w, const Box& b, const Box& b0) const {
         if (threadIdx.x & 31) return;
         const Node& s = w.node;
         float dh[3], dl[3], sh[3], sl[3];
         for (int q = 0; q < 3; ++q) {
-            df_diff(b0.c[2 * q], b0.c[2 * q + 1], s.c[2 * q], s.c[2 * q + 1], dh[q], dl[q]);
+            const Box& o = q == b.ax1 || q == b.ax2 ? b0 : b;
+            df_diff(o.c[2 * q], o.c[2 * q + 1], s.c[2 * q], s.c[2 * q + 1], dh[q], dl[q]);
             df_sqr(dh[q], dl[q], sh[q], sl[q]);
         }
         df_add_pos(sh[0], sl[0], sh[1], sl[1], sh[0], sl[0]);

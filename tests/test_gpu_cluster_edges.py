@@ -1,0 +1,100 @@
+"""The clustered sums (stage_cluster.cu, raytrace.cu) on target sets and
+amplitudes that the other tests do not have.
+
+Tolerance against FP64 as in test_gpu_cluster.py: 5e-6 beyond the direct
+sum's own error, here with the worst value bounded as well."""
+import math
+
+import pytest
+import torch
+
+from fieldcheck import assert_close, rel_l2
+from paper_2408_06765_gb300 import build, rsi, workloads
+
+pytestmark = pytest.mark.gpu
+TOL = 5e-6
+K_WATER, K_STEEL = (2 * math.pi * 2e6 / c for c in (1480.0, 5900.0))
+
+
+@pytest.fixture(scope="module", autouse=True)
+def lib():
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    build.build()
+
+
+def disk(n, tilt=0.0):
+    return rsi.make_qmc_points({"kind": "disk", "centre": (0.0, 0.0, 0.0), "a": 6.35e-3, "tilt": tilt}, 3, 0, n)
+
+
+def interface(n, z=0.05, w=0.03):
+    return rsi.make_qmc_points({"kind": "rect", "centre": (0.0, 0.0, z), "wx": w, "wy": w}, 3, 1, n)
+
+
+def image(nx, nz, z0, z1, half=0.02):
+    return rsi.grid_points({"x0": -half, "x1": half, "nx": nx, "z0": z0, "z1": z1, "nz": nz})
+
+
+def points(x, y, z):
+    """A target set of a caller's own coordinates (float64 tensors), in the order given."""
+    pts = rsi.Points(x.numel())
+    pts.buf.zero_()
+    for name, v in (("X", x), ("Y", y), ("Z", z)):
+        set_coordinate(pts, name, slice(None), v.reshape(-1).cuda())
+    return pts
+
+
+def set_coordinate(pts, name, at, v):
+    hi = torch.as_tensor(v, dtype=torch.float64).to(torch.float32)
+    pts.field(name)[at] = v
+    pts.field(name + "H")[at] = hi.cuda()
+    pts.field(name + "L")[at] = (torch.as_tensor(v, dtype=torch.float64) - hi.double()).float().cuda()
+
+
+def volume(nx, ny, nz, step, z0, slow=("z", "y")):
+    """A box of targets, x fastest, then y and z, or z and y."""
+    ax = {"x": (torch.arange(nx, dtype=torch.float64) - nx / 2) * step,
+          "y": (torch.arange(ny, dtype=torch.float64) - ny / 2) * step,
+          "z": torch.arange(nz, dtype=torch.float64) * step + z0}
+    c = dict(zip(slow + ("x",), torch.meshgrid(*(ax[a] for a in slow + ("x",)), indexing="ij")))
+    return points(c["x"], c["y"], c["z"])
+
+
+def stage_fields(kind, k, src, sigma, tgt):
+    return [rsi.propagate_stage(rsi.stage_struct(kind, prec, k, variant=var), src, sigma, tgt)
+            for prec, var in (("fp64", 0), ("fp32c", 3), ("fp32c", 0))]
+
+
+# Targets in rows of which a block of 1024 spans two planes and a quarter of it
+# one: strips of 32 slices of a volume, two rows of y each; images 48 rows high
+# one behind the other in y, 8 and 1 mm apart; all against a tilted piston and
+# an interface below which they lie.
+SETS = {
+    "volume": lambda: volume(48, 32, 64, 0.5e-3, 0.06),
+    "images": lambda: volume(128, 8, 48, 0.25e-3, 0.07, slow=("y", "z")),
+    "thin stack": lambda: volume(256, 5, 48, 0.1e-3, 0.08, slow=("y", "z")),
+}
+
+
+@pytest.mark.parametrize("kind", ["piston", "interface"])
+@pytest.mark.parametrize("name", list(SETS))
+def test_targets_off_a_plane_match_fp64(name, kind):
+    tgt = SETS[name]()
+    if kind == "piston":
+        exact, direct, got = stage_fields(rsi.STAGE_PISTON, K_WATER, disk(16384, 0.1), None, tgt)
+    else:
+        src = interface(65536)
+        sigma = rsi.propagate_stage(rsi.stage_struct(rsi.STAGE_PISTON, "fp32c", K_WATER, variant=3), disk(4096), None, src)
+        exact, direct, got = stage_fields(rsi.STAGE_RSI, K_STEEL, src, sigma, tgt)
+    rsi.sync_status()
+    own = rel_l2(direct.cpu(), exact.cpu())
+    assert_close(got.cpu(), exact.cpu(), own + TOL, name)
+
+
+@pytest.mark.parametrize("first,count", [(37, 128 * 300), (300, 40001), (128 * 64, 128 * 256)])
+def test_slices_of_an_image_match_fp64(first, count):
+    """A share of an image's slots, from within a row or in ragged numbers."""
+    tgt = rsi.points_slice(image(128, 512, 0.05, 0.09), first, count)
+    exact, direct, got = stage_fields(rsi.STAGE_PISTON, K_WATER, disk(20011, 0.1), None, tgt)
+    rsi.sync_status()
+    assert not torch.equal(got, direct)  # the clustered kernel ran
+    assert_close(got.cpu(), exact.cpu(), rel_l2(direct.cpu(), exact.cpu()) + TOL)
