@@ -194,7 +194,9 @@ __device__ __forceinline__ RayRef ray_reference(float qxh, float qxl, float qyh,
     float x = __fmaf_rn(-n, a.tp.p1, ph);
     x = __fmaf_rn(-n, a.tp.p2, x);
     x = __fmaf_rn(-n, a.tp.p3, x);
-    R.tau = __fadd_rn(x, pl);
+    // df_sqrt takes what is not a number for 0: such a foot makes the phase one, so
+    // that the sum is reported
+    R.tau = __fmaf_rn(0.0f, __fadd_rn(dxh, dyh), __fadd_rn(x, pl));
     return R;
 }
 

@@ -1092,15 +1092,20 @@ __device__ __forceinline__ void make_boxes(const TgtView& tgt, int64_t n_tgt, in
     const int64_t jr = strip_slot(t0, n_tgt, L, h);  // all offsets from the block's first target
     const float rh[3] = {tgt.xh[jr], tgt.yh[jr], tgt.zh[jr]}, rl[3] = {tgt.xl[jr], tgt.yl[jr], tgt.zl[jr]};
     float p[TPT][3], lo, ext[6];
+    int wrong = 0;  // bit q: a target of quarter q has a coordinate that is not a number
 #pragma unroll
     for (int q = 0; q < TPT; ++q) {
         df_diff(tgt.xh[j[q]], tgt.xl[j[q]], rh[0], rl[0], p[q][0], lo);
         df_diff(tgt.yh[j[q]], tgt.yl[j[q]], rh[1], rl[1], p[q][1], lo);
         df_diff(tgt.zh[j[q]], tgt.zl[j[q]], rh[2], rl[2], p[q][2], lo);
+        if (!(isfinite(p[q][0]) && isfinite(p[q][1]) && isfinite(p[q][2]))) wrong |= 1 << q;
     }
     int ax3 = 0;
     float whole[6];
     for (int b = 0; b < (TPT > 1 ? 1 + TPT : 1); ++b) {
+        // minima pass over NaN, and the clustered sum does not read a target's third
+        // coordinate: such a rectangle is left to the direct sum, which reports it
+        const bool numbers = !__syncthreads_or(b == 0 ? wrong : wrong & (1 << (b - 1)));
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
             float a = INFINITY, c = INFINITY;
@@ -1127,7 +1132,7 @@ __device__ __forceinline__ void make_boxes(const TgtView& tgt, int64_t n_tgt, in
                 wm[d] = 0.5f * (whole[d] - whole[3 + d]);
                 df_diff(rh[d], rl[d], -mid[d], 0.0f, o.c[2 * d], o.c[2 * d + 1]);
             }
-            o.q1 = half[o.ax1], o.q2 = half[o.ax2], o.q3 = half[ax3];
+            o.q1 = half[o.ax1], o.q2 = half[o.ax2], o.q3 = numbers ? half[ax3] : INFINITY;
             o.o1 = o.q1 > 0.0f ? (wm[o.ax1] - mid[o.ax1]) / o.q1 : 0.0f;
             o.o2 = o.q2 > 0.0f ? (wm[o.ax2] - mid[o.ax2]) / o.q2 : 0.0f;
             out[b] = o;

@@ -98,3 +98,27 @@ def test_slices_of_an_image_match_fp64(first, count):
     rsi.sync_status()
     assert not torch.equal(got, direct)  # the clustered kernel ran
     assert_close(got.cpu(), exact.cpu(), rel_l2(direct.cpu(), exact.cpu()) + TOL)
+
+
+@pytest.mark.parametrize("value", [math.nan, math.inf, -math.inf])
+@pytest.mark.parametrize("coordinate", ["X", "Y", "Z"])
+@pytest.mark.parametrize("kind", ["piston", "raytrace"])
+def test_a_target_that_is_no_number_is_reported(kind, coordinate, value):
+    """... and leaves every other target as it was."""
+    tgt, at = image(256, 256, 0.06, 0.10), 256 * 100 + 37
+    if kind == "piston":
+        src = disk(16384)
+        run = lambda: rsi.propagate_stage(rsi.stage_struct(rsi.STAGE_PISTON, "fp32c", K_WATER), src, None, tgt)
+    else:
+        cfg = workloads.f2_ray_tracing(n_piston=16384, nx=256, nz=256)
+        src, tgt = disk(16384), rsi.grid_points(cfg["grid"])
+        run = lambda: rsi.raytrace_field(rsi.raytrace_struct(cfg), src, tgt)
+    want = run()
+    rsi.sync_status()
+    set_coordinate(tgt, coordinate, at, value)
+    got = run()
+    with pytest.raises(rsi.RSIError):
+        rsi.sync_status()
+    assert not torch.isfinite(torch.view_as_real(got[at])).all()
+    got[at] = want[at]
+    assert rel_l2(got.cpu(), want.cpu()) <= TOL
