@@ -450,7 +450,11 @@ __device__ __forceinline__ void warp_item(const M& model, const Sum& g, const Bo
         const float3 p = make_float3(fmaf(s1, s.e1[0], s2 * s.e2[0]), fmaf(s1, s.e1[1], s2 * s.e2[1]),
                                      fmaf(s1, s.e1[2], s2 * s.e2[2]));
         // m e^{i beta} with beta in [-pi/2, pi/2]: a negated moment negates m alone
-        float m = sqrtf(fmaf(m2.x, m2.x, m2.y * m2.y));
+        // the modulus over a power of two, since the squares of amplitudes in a small or
+        // a large unit leave FP32's range where the amplitudes do not
+        const int e = min(max((__float_as_int(fmaxf(fabsf(m2.x), fabsf(m2.y))) >> 23), 1), 253);
+        const float up = __int_as_float((254 - e) << 23), mx = up * m2.x, my = up * m2.y;
+        float m = __int_as_float(e << 23) * sqrtf(fmaf(mx, mx, my * my));
         if (m2.x < 0.0f || (m2.x == 0.0f && m2.y < 0.0f)) m = -m, m2.x = -m2.x, m2.y = -m2.y;
         model.node_record(b, rc, p, m, atan2f(m2.y, m2.x), w.rows + (o >> 1) * 16 + (o & 1));
     }

@@ -122,3 +122,30 @@ def test_a_target_that_is_no_number_is_reported(kind, coordinate, value):
     assert not torch.isfinite(torch.view_as_real(got[at])).all()
     got[at] = want[at]
     assert rel_l2(got.cpu(), want.cpu()) <= TOL
+
+
+@pytest.mark.parametrize("kind", ["piston", "interface", "raytrace"])
+@pytest.mark.parametrize("power", [-80, -60, 60, 80])
+def test_fields_are_linear_in_the_amplitude(kind, power):
+    """A power of two of the velocity or density is one of the field.  Every
+    product and sum of the kernel keeps its bits under it as long as nothing
+    leaves the range of FP32; the smallest moments' parts do at 2^-80, by
+    2^-149 / 2^-110 of the largest."""
+    s = 2.0 ** power
+
+    def run(s):
+        if kind == "piston":
+            st = rsi.stage_struct(rsi.STAGE_PISTON, "fp32c", K_WATER, s)
+            return rsi.propagate_stage(st, disk(16384), None, image(256, 256, 0.06, 0.10))
+        if kind == "interface":
+            src = interface(65536)
+            sigma = torch.full((src.n,), s, dtype=torch.complex128, device="cuda")
+            return rsi.propagate_stage(rsi.stage_struct(rsi.STAGE_RSI, "fp32c", K_STEEL), src, sigma, image(256, 192, 0.07, 0.11))
+        cfg = workloads.f2_ray_tracing(n_piston=16384, nx=256, nz=256)
+        cfg["v0"] = s
+        return rsi.raytrace_field(rsi.raytrace_struct(cfg), disk(16384), rsi.grid_points(cfg["grid"]))
+
+    one, got = run(1.0), run(s)
+    rsi.sync_status()
+    assert float(torch.linalg.vector_norm(got)) > 0.0
+    assert_close((got / s).cpu(), one.cpu(), 1e-7)
