@@ -197,8 +197,9 @@ size_t rsi_stage_workspace_bytes(const rsi_stage *st, int64_t n_src, int64_t n_t
  * src_sigma: complex [n_src] in the source set's slot order (RSI only; NULL
  * for PISTON).  tgt_field: complex [n_tgt] in the target set's slot order,
  * overwritten.  workspace: >= rsi_stage_workspace_bytes(...), 256-byte
- * aligned; its contents are scratch.  Calls that share a workspace must be
- * ordered on one stream.                                                   */
+ * aligned; its contents are scratch.  One without room for the clusters' tables
+ * but for the direct sum (the size for variant 3) gets the direct sum.  Calls
+ * that share a workspace must be ordered on one stream.                     */
 int rsi_propagate_stage(const rsi_stage *st,
                         const void *src_points, int64_t n_src, const double *src_sigma,
                         const void *tgt_points, int64_t n_tgt, double *tgt_field,

@@ -909,6 +909,7 @@ extern "C" int rsi_raytrace_field(const rsi_raytrace* rt, const void* src_points
     RtPlan p;
     int rc = rt_plan(*rt, n_src, n_tgt, p);
     if (rc != RSI_OK) return rc;
+    if (workspace_bytes < p.bytes()) p.clustered = false;  // room for the direct sum alone
     if (workspace_bytes < p.bytes())
         return rsi_fail(RSI_E_NOMEM, "rsi_raytrace_field: workspace %zu < %zu bytes", workspace_bytes, p.bytes());
     int* status = rsi_status_ptr();

@@ -244,6 +244,7 @@ extern "C" int rsi_propagate_stage(const rsi_stage* st, const void* src_points, 
     Plan p;
     int rc = make_plan(*st, n_src, n_tgt, p);
     if (rc != RSI_OK) return rc;
+    if (workspace_bytes < p.bytes()) p.clustered = false;  // room for the direct sum alone
     if (workspace_bytes < p.bytes())
         return rsi_fail(RSI_E_NOMEM, "rsi_propagate_stage: workspace %zu < %zu bytes", workspace_bytes, p.bytes());
     int* status = rsi_status_ptr();

@@ -249,7 +249,9 @@ bool cluster_plan(int kind, int normals, int nf, int64_t n_src, int64_t n_tgt, i
     p.segs = int(std::max<int64_t>(1, std::min<int64_t>({std::max<int64_t>(16, 608 / blocks), n_tiles / 4,
                                                          (int64_t(1) << 24) / n_tgt})));
     p.partial_bytes = align256(size_t(p.splits + p.segs) * size_t(n_tgt) * sizeof(double2));
-    return true;
+    // 32 GiB of tables, an eighth of the GPU's memory, are the most that is asked
+    // for beside the point sets: the mask's byte per block and tile reaches it at 9e15 pairs
+    return double(p.extra_bytes) + double(nf) * double(p.partial_bytes) <= 0x1p35;
 }
 
 int cluster_prepare(const rsi_stage& st, const double* ks, float gate_ratio, const PointsView& src, int64_t n_src,

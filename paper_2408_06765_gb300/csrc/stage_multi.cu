@@ -899,6 +899,7 @@ extern "C" int rsi_propagate_stage_multi(const rsi_stage* st, int32_t nf, const 
     MultiArgs a = {};
     int rc = mplan(*st, nf, ks, n_src, n_tgt, p, a);
     if (rc != RSI_OK) return rc;
+    if (workspace_bytes < p.bytes()) p.clustered = false;  // room for the direct sum alone
     if (workspace_bytes < p.bytes())
         return rsi_fail(RSI_E_NOMEM, "rsi_propagate_stage_multi: workspace %zu < %zu bytes", workspace_bytes,
                         p.bytes());

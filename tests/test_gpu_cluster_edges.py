@@ -3,6 +3,7 @@ amplitudes that the other tests do not have.
 
 Tolerance against FP64 as in test_gpu_cluster.py: 5e-6 beyond the direct
 sum's own error, here with the worst value bounded as well."""
+import ctypes
 import math
 
 import pytest
@@ -149,3 +150,48 @@ def test_fields_are_linear_in_the_amplitude(kind, power):
     rsi.sync_status()
     assert float(torch.linalg.vector_norm(got)) > 0.0
     assert_close((got / s).cpu(), one.cpu(), 1e-7)
+
+
+@pytest.mark.parametrize("kind", ["piston", "several frequencies", "raytrace"])
+def test_a_workspace_for_the_direct_sum_gets_the_direct_sum(kind):
+    """A scratch buffer of the direct sum's size, and nothing smaller."""
+    lib, src, tgt = rsi.load(), disk(16384), image(256, 256, 0.06, 0.10)
+    out = torch.empty((3, tgt.n), dtype=torch.complex128, device="cuda")
+    ks = (ctypes.c_double * 3)(K_WATER, 1.3 * K_WATER, 1.7 * K_WATER)
+    cfg = workloads.f2_ray_tracing(n_piston=16384, nx=256, nz=256)
+    if kind == "raytrace":
+        tgt = rsi.grid_points(cfg["grid"])
+    stream = rsi._stream()
+
+    def call(ask, nbytes=None):
+        """The size asked for, or the call with a buffer of so many bytes."""
+        if kind == "raytrace":
+            st = rsi.raytrace_struct(cfg, tile=256 if ask else 0)
+            args = (src.ptr(), src.n, tgt.ptr(), tgt.n, rsi._ptr(out))
+            size, run = lib.rsi_raytrace_workspace_bytes(ctypes.byref(st), src.n, tgt.n), lib.rsi_raytrace_field
+        else:
+            st = rsi.stage_struct(rsi.STAGE_PISTON, "fp32c", K_WATER, variant=3 if ask else 0)
+            args = (src.ptr(), src.n, None, tgt.ptr(), tgt.n, rsi._ptr(out))
+            if kind == "piston":
+                size, run = lib.rsi_stage_workspace_bytes(ctypes.byref(st), src.n, tgt.n), lib.rsi_propagate_stage
+            else:
+                size = lib.rsi_stage_multi_workspace_bytes(ctypes.byref(st), 3, ks, src.n, tgt.n)
+                run, args = lib.rsi_propagate_stage_multi, (3, ks) + args
+        if nbytes is None:
+            return size
+        ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+        out.fill_(0)
+        rc = run(ctypes.byref(st), *args, rsi._ptr(ws), nbytes, stream)
+        return rc, out.clone()
+
+    small, large = call(True), call(False)
+    assert small < large
+    rc, want = call(True, small)
+    assert rc == 0
+    for nbytes in (small, large - 1):
+        rc, got = call(False, nbytes)
+        assert rc == 0 and torch.equal(got, want)
+    rc, got = call(False, large)
+    assert rc == 0 and not torch.equal(got, want)
+    assert call(False, small - 1)[0] == -5  # RSI_E_NOMEM
+    rsi.sync_status()
