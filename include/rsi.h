@@ -326,7 +326,7 @@ size_t rsi_raytrace_workspace_bytes(const rsi_raytrace *rt, int64_t n_src, int64
  * on the wrong side of the interface break the model: their sums come out
  * non-finite (recorded in the status word).  Same conventions for point
  * sets, field, workspace and stream as rsi_propagate_stage.  With tile and
- * newton 0, sums of 3e8 pairs and more may take far clusters of points through
+ * newton 0, sums of 3.4e8 pairs and more may take far clusters of points through
  * Chebyshev nodes, chosen on the device, as rsi_propagate_stage does.       */
 int rsi_raytrace_field(const rsi_raytrace *rt, const void *src_points, int64_t n_src,
                        const void *tgt_points, int64_t n_tgt, double *tgt_field,

@@ -43,8 +43,10 @@ struct StageGate {
 // much slower it issues them than the direct kernel (estimate()), and those of
 // the direct sums it leaves; against the direct kernel's 16.8 per 32 pairs, 256
 // S pairs per sample.  `ratio`: a multi-frequency stage's instructions per
-// frequency, or a ray's per pair, over a single stage's.  FP32 arithmetic on
-// integers: the same in every thread of both kernels.
+// frequency, or a ray's per pair, over a single stage's, and the share of the
+// direct sum's time that is left beside the clustered kernel's own
+// (cluster_plan()).  FP32 arithmetic on integers: the same in every thread of both
+// kernels.
 __device__ __forceinline__ bool gate_clustered(const StageGate* g, int S, float ratio) {
     return float(g->cost) * 1.05f < float(g->pairs) * (134.4f * float(S)) * ratio;
 }

@@ -175,18 +175,21 @@ size_t nodes_bytes(int n_tiles) {
 
 }  // namespace
 
-// Clusters pay where the sum is long: preparation, estimate and the launches take
-// about 40 us more than the direct kernel's, and 6e8 pairs take that kernel
-// 0.45 ms.  A piston's clusters are small beside the distance and nearly always
-// taken; an interface's may not be, so its sums have to be longer, and those of
-// several frequencies, whose direct sum is shared, two or three times as long (9e8
-// and 7.8e8 pairs at three frequencies: no faster, and 40 us lost);
-// a ray costs the direct kernel 7 times a stage's pair (16384 x 256 x 128:
-// 2.32 -> 1.81 ms, 9001 x 101 x 77: 0.55 -> 1.29 ms).  Per-point normals turn within a
-// tile on every curved surface, where the direct sum would be taken anyway.
+// Clusters pay where the sum is long.  Where the device's estimate decides for the
+// direct sum, its launches and the preparation cost 35 us, 8% of a sum of 5e8
+// pairs and 4% of one of 1e9.  Random sums, speed with clusters offered over
+// without (geometric mean): piston 5e8 .. 6e8 pairs 0.94 (single ones up to 3.9),
+// 6e8 .. 7.5e8 1.05, 1e9 .. 1.5e9 1.17; interface 1e9 .. 1.5e9 1.10, 1.5e9 .. 2.5e9
+// 1.33.  A piston's clusters are small beside the distance and mostly taken; an
+// interface's may not be, so its sums have to be longer, and those of several
+// frequencies, whose direct sum is shared, two or three times as long (9e8 and
+// 7.8e8 pairs at three frequencies: no faster, and 40 us lost).  A ray costs the
+// direct kernel 7 times a stage's pair: 3e8 .. 3.4e8 pairs 0.84, 4e8 .. 5e8 1.07,
+// 5e8 .. 6e8 1.17.  Per-point normals turn within a tile on every curved surface,
+// where the direct sum would be taken anyway.
 bool cluster_plan(int kind, int normals, int nf, int64_t n_src, int64_t n_tgt, int S, int splits, int max_auto_splits,
                   ClusterPlan& p) {
-    const double least = kind == RSI_TIMING_RAYTRACE ? 3e8
+    const double least = kind == RSI_TIMING_RAYTRACE ? 3.4e8
                          : kind == RSI_STAGE_PISTON   ? (nf > 1 ? 1e9 : 5e8)
                                                       : (nf > 1 ? 3e9 : 1e9);
     if (n_src < 8192 || n_tgt < 4096 || double(n_src) * double(n_tgt) < least) return false;
@@ -232,11 +235,18 @@ bool cluster_plan(int kind, int normals, int nf, int64_t n_src, int64_t n_tgt, i
     // 0.64; interface 120000 onto 9 0.90, 1.01, but 262144 onto 5, 64 roots for
     // their CTAs, 1.04, 0.76 and 65536 onto 16 0.88, 0.75; rays from 16384 onto 32 2.32, 1.77
     if (blocks < (kind == RSI_STAGE_PISTON ? 32 : 16) && roots < 64) return false;
-    // what the 60 us of launches and CTAs' set-up, at 9.2e11 instructions per warp
-    // and second, leave of the direct sum's time for the clusters' arithmetic
-    // (134.4 instructions per source and 256 targets)
-    const double direct = (kind == RSI_TIMING_RAYTRACE ? 976.0 : 134.4) * double(n_src) * double(blocks * kTpt) * nf;
-    p.gain = float(std::max(0.0, 1.0 - 5.5e7 / direct));
+    // The share of the direct sum's time (134.4 instructions per source and 256
+    // targets, 9.2e11 per warp and second) that the estimate may reach: what is left
+    // beside the preparation, the launches and the last CTAs, which end up to 0.2 ms
+    // after the work is used up, for rays from tiles of 128 points 0.85 ms, over how
+    // far the CTAs' own times lie above the estimate.  Fitted to 1600 random sums:
+    // with 0.06 ms and 1 for all of them 184 went to a kernel more than 3% slower (the
+    // worst 1.55 times), now 58 (the worst 1.30 times); 12 that clusters would speed
+    // up by more than 5% keep the direct sum.
+    const bool ray = kind == RSI_TIMING_RAYTRACE, piston = kind == RSI_STAGE_PISTON;
+    const double direct = (ray ? 976.0 : 134.4) * double(n_src) * double(blocks * kTpt) * nf;
+    const double ms = ray ? (S < 256 ? 0.85 : 0.19) : piston ? 0.16 : 0.2;
+    p.gain = float(std::max(0.0, 1.0 - ms * 9.2e8 / direct) / (ray ? 1.0 : piston ? 1.2 : 1.05));
     p.tile_bytes = RSI_TILE_HDR_BYTES + size_t(S) * fp32_record_bytes(kind, base_normals(normals));
     p.tiles_bytes = align256(size_t(n_tiles) * p.tile_bytes);
     p.boxes_at = nodes_bytes(n_tiles);

@@ -195,3 +195,22 @@ def test_a_workspace_for_the_direct_sum_gets_the_direct_sum(kind):
     assert rc == 0 and not torch.equal(got, want)
     assert call(False, small - 1)[0] == -5  # RSI_E_NOMEM
     rsi.sync_status()
+
+
+@pytest.mark.parametrize("n,nx,nz", [(19000, 129, 127), (9300, 256, 128)])
+def test_short_ray_sums_take_the_direct_kernel(n, nx, nz):
+    """3e8 rays: the clustered sum took 1.1 to 1.3 times as long."""
+    cfg = workloads.f2_ray_tracing(n_piston=n, nx=nx, nz=nz)
+    got, direct = rsi.run_raytrace(cfg), rsi.run_raytrace(cfg, tile=128 if n < 16384 else 256)
+    rsi.sync_status()
+    assert torch.equal(got, direct)
+
+
+def test_a_short_sum_close_to_its_interface_takes_the_direct_kernel():
+    """1e9 pairs, most clusters too close: the clustered sum took 1.14 times as long."""
+    k, src, tgt = 2 * math.pi * 5e6 / 5900.0, interface(61100), image(128, 128, 0.0505, 0.09)
+    sigma = torch.ones(src.n, dtype=torch.complex128, device="cuda")
+    got, direct = (rsi.propagate_stage(rsi.stage_struct(rsi.STAGE_RSI, "fp32c", k, variant=v), src, sigma, tgt)
+                   for v in (0, 3))
+    rsi.sync_status()
+    assert torch.equal(got, direct)
