@@ -222,7 +222,7 @@ int rsi_propagate_stage(const rsi_stage *st,
  * frequency twice another), e^{i k_j (r - R)} is formed from e^{i k_i (r - R)}
  * by the double angle on pairs away from the tile, two MUFU operations per
  * pair fewer (in the direct sum; clusters, as in rsi_propagate_stage, are taken
- * frequency by frequency).  The doubled angle carries twice the sincos's angle error: on
+ * frequency by frequency; a variant, tile or tpt asks for the direct sum).  The doubled angle carries twice the sincos's angle error: on
  * 2.25, 5 and 10 MHz the 10 MHz image is 9.7e-7 from the FP64 oracle (5.5e-7
  * with its own sincos), far inside the FP32C tolerance.                    */
 size_t rsi_stage_multi_workspace_bytes(const rsi_stage *st, int32_t nf, const double *ks, int64_t n_src,

@@ -605,13 +605,17 @@ def run_chain_multi(cfgs: list, fmt: str = "c128", workspace: Workspace | None =
                     stage_opts: dict | None = None, stream=None, device="cuda") -> list:
     """The chains of 2-4 workloads that differ only in frequency, every stage
     evaluated for all frequencies at once (rsi_propagate_stage_multi).
-    Returns one image per workload, as run_chain would."""
+    Returns one image per workload, as run_chain would.  stage_opts: the launch
+    shape of every stage; any tile, tpt or variant asks for the direct sums
+    (variants 1 and 2 for the packed ones too, as 3 does)."""
     if not same_geometry(cfgs) or not 2 <= len(cfgs) <= 4:
         raise ValueError("run_chain_multi needs 2-4 workloads that differ only in frequency")
     cfg = cfgs[0]
     if cfg.get("precision", "fp32c") != "fp32c":
         raise ValueError("run_chain_multi is FP32C only")
-    opts = {k: v for k, v in (stage_opts or {}).items() if k != "variant"}
+    opts = dict(stage_opts or {})
+    if opts.get("variant"):
+        opts["variant"] = 3
     ws = workspace or Workspace(device)
     seed = int(cfg.get("seed", 0))
     v0 = float(cfg.get("v0", 1.0))

@@ -214,3 +214,19 @@ def test_a_short_sum_close_to_its_interface_takes_the_direct_kernel():
                    for v in (0, 3))
     rsi.sync_status()
     assert torch.equal(got, direct)
+
+
+@pytest.mark.parametrize("variant", [1, 2, 3])
+def test_a_variant_asks_for_the_direct_sums_of_several_frequencies(variant):
+    cfgs = []
+    for f in (2e6, 3e6):
+        cfg = workloads.c2_full_image(f)
+        cfg["piston"]["n"], cfg["interfaces"][0]["n"] = 16384, 65536
+        cfg["grid"].update({"nx": 256, "nz": 192})
+        cfgs.append(cfg)
+    got = rsi.run_chain_multi(cfgs, stage_opts={"variant": variant})
+    want = rsi.run_chain_multi(cfgs, stage_opts={"tile": 256})
+    clustered = rsi.run_chain_multi(cfgs)
+    rsi.sync_status()
+    for a, b, c in zip(got, want, clustered):
+        assert torch.equal(a, b) and not torch.equal(a, c)
