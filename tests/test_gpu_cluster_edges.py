@@ -230,3 +230,26 @@ def test_a_variant_asks_for_the_direct_sums_of_several_frequencies(variant):
     rsi.sync_status()
     for a, b, c in zip(got, want, clustered):
         assert torch.equal(a, b) and not torch.equal(a, c)
+
+
+@pytest.mark.parametrize("kind,freqs", [
+    ("piston", (1e6, 1.7e6, 2e6)), ("interface", (1e6, 1.7e6)), ("interface", (1e6, 1.7e6, 2e6)),
+    ("interface", (1e6, 1.3e6, 1.7e6, 1.9e6)),
+])
+def test_several_frequencies_take_clusters_and_match_fp64(kind, freqs):
+    """Each frequency with a density of its own; three of them with and four
+    without one that is twice another."""
+    ks = [2 * math.pi * f / (1480.0 if kind == "piston" else 5900.0) for f in freqs]
+    if kind == "piston":
+        src, sigma, tgt, what = disk(16384), None, image(256, 256, 0.06, 0.10), rsi.STAGE_PISTON
+    else:
+        src, tgt, what = interface(65536), image(256, 192, 0.07, 0.11), rsi.STAGE_RSI
+        sigma = torch.stack([rsi.propagate_stage(rsi.stage_struct(rsi.STAGE_PISTON, "fp32c", 2 * math.pi * f / 1480.0, variant=3),
+                                                 disk(4096), None, src) for f in freqs])
+    got, direct = (rsi.propagate_stage_multi(rsi.stage_struct(what, "fp32c", ks[0], variant=v), ks, src, sigma, tgt)
+                   for v in (0, 3))
+    rsi.sync_status()
+    for f, k in enumerate(ks):
+        exact = rsi.propagate_stage(rsi.stage_struct(what, "fp64", k), src, None if sigma is None else sigma[f], tgt)
+        assert not torch.equal(got[f], direct[f])
+        assert_close(got[f].cpu(), exact.cpu(), rel_l2(direct[f].cpu(), exact.cpu()) + TOL, f"{freqs[f]:g} Hz")
