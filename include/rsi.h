@@ -339,7 +339,8 @@ enum rsi_image_format {
     RSI_IMG_ABS32 = 2 /* float |k phi / v0| [nz][nx]                            */
 };
 /* out[j] = (k / v0) field[j] for the grid's nx*nz pixels (normalised
- * velocity amplitude k phi / v0 of Fig. oblique_incidence).                */
+ * velocity amplitude k phi / v0 of Fig. oblique_incidence).  field: 16-byte
+ * aligned; out: aligned to the format's pixels.                            */
 int rsi_field_image(const rsi_grid *g, const double *field, double k, double v0,
                     int32_t format, void *out, void *stream);
 /* out[j] = (k / v0) (field_a[j] + field_b[j]): the image of a medium holding

@@ -86,9 +86,11 @@ extern "C" int rsi_field_image_sum(const rsi_grid* g, const double* field, const
     if (format < RSI_IMG_C128 || format > RSI_IMG_ABS32)
         return rsi_fail(RSI_E_INVAL, "rsi_field_image: unknown format %d", format);
     if (!(v0 != 0.0)) return rsi_fail(RSI_E_INVAL, "rsi_field_image: v0 must be non-zero");
+    // pixels are written one by one, so that an image may begin at any pixel of another
+    const size_t pixel = format == RSI_IMG_C128 ? 16 : format == RSI_IMG_C64 ? 8 : 4;
     if (reinterpret_cast<uintptr_t>(field) % 16 || reinterpret_cast<uintptr_t>(field_b) % 16 ||
-        reinterpret_cast<uintptr_t>(out) % 16)
-        return rsi_fail(RSI_E_INVAL, "rsi_field_image: arrays must be 16-byte aligned");
+        reinterpret_cast<uintptr_t>(out) % pixel)
+        return rsi_fail(RSI_E_INVAL, "rsi_field_image: fields must be 16-byte aligned, the image to its pixels' size");
     int64_t n = int64_t(g->nx) * g->nz;
     int threads = 256;
     unsigned blocks = unsigned((n + threads - 1) / threads);

@@ -102,3 +102,16 @@ def test_two_medium_full_size_matches_stored_oracle():
     got = res.image.reshape(-1).cpu().numpy()[np.asarray(rec["pixels"])]
     want = np.asarray(rec["re"]) + 1j * np.asarray(rec["im"])
     assert_close(got, want, 1e-4)
+
+
+@pytest.mark.parametrize("fmt,tol", [("c64", 6e-8), ("abs32", 6e-8)])
+def test_windows_of_an_odd_number_of_pixels(fmt, tol):
+    """The second window then begins off 16 bytes of the shared image: the same
+    pixels, each rounded to the format (2^-24) once."""
+    cfg = W.f1_two_medium(n_piston=500, n_iface=1000, nx=37, nz_water=29, nz_solid=31)
+    want = rsi.run_two_medium(cfg).image
+    got = rsi.run_two_medium(cfg, fmt=fmt).image
+    rsi.sync_status()
+    want = want if fmt == "c64" else want.abs()
+    assert got.shape == want.shape
+    assert float(((got.to(want.dtype) - want).abs() / want.abs()).max()) <= tol
