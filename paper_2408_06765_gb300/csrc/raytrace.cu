@@ -775,7 +775,7 @@ __global__ void __launch_bounds__(rsi_cluster::kThreads)
     for (int l = 0; l < kLevels; ++l) {
         if (b < count) {
             const int64_t i0 = b * len, i1 = i0 + len < c.n_src ? i0 + len : c.n_src;
-            make_node(RSI_STAGE_PISTON, RSI_NORMALS_Z, c.src, c.n_src, mode, i0, i1, nodes + b, red);
+            make_node(RSI_STAGE_PISTON, c.src, c.n_src, mode, i0, i1, nodes + b, red);
             return;
         }
         b -= count;

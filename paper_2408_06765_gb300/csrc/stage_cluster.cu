@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(kThreads) cluster_prep_kernel(const __grid_con
     for (int l = 0; l < kLevels; ++l) {
         if (b < count) {
             const int64_t i0 = b * len, i1 = i0 + len < a.n_src ? i0 + len : a.n_src;
-            make_node(a.kind, a.normals, a.src, a.n_src, mode, i0, i1, nodes + b, red);
+            make_node(a.kind, a.src, a.n_src, mode, i0, i1, nodes + b, red);
             return;
         }
         b -= count;

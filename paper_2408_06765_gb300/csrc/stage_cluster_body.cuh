@@ -17,7 +17,7 @@
 // Sources are clustered in tiles (256), groups of 4 tiles and of 16 tiles,
 // targets in blocks of 1024 and their quarters; each pair is taken at the
 // coarsest level that choose_nodes() admits, and pairs of a tile and a quarter
-// that it does not admit (too close, thick, or with turning normals) take the
+// that it does not admit (too close or thick) take the
 // direct sum (stage_fp32_body.cuh).
 //
 // Accuracy.  The phases of sources and targets are formed as the direct sum
@@ -48,7 +48,7 @@ struct Node {
     float c[6];            // centre of its rectangle, (hi, lo) per axis
     float e1[3], e2[3], e3[3];  // unit axes; e3 is the plane's normal
     float h1, h2, h3;      // half sizes along them
-    float flat;            // 1: the sources' obliquity normal is e3 everywhere
+    float flat;            // 1: every coordinate is a number (the obliquity's normal is e3 everywhere)
     float pad[13];
 };
 static_assert(sizeof(Node) == 128, "node");
@@ -964,14 +964,14 @@ __device__ __forceinline__ void sum_block_order(const double2* __restrict__ part
 // preparation
 // ---------------------------------------------------------------------------
 // Frame and rectangle of sources [i0, i1) (in the order of `mode`) of a set; one CTA.
-__device__ __forceinline__ void make_node(int kind, int normals, const PointsView& src, int64_t n, int mode,
-                                          int64_t i0, int64_t i1, Node* out, float* red) {
+__device__ __forceinline__ void make_node(int kind, const PointsView& src, int64_t n, int mode, int64_t i0, int64_t i1,
+                                          Node* out, float* red) {
     const int64_t first = rsi_fp32::source_slot(i0, n, mode);
     const float xh = src.xh[first], xl = src.xl[first], yh = src.yh[first], yl = src.yl[first], zh = src.zh[first],
                 zl = src.zl[first];
-    // plane normal: the obliquity's own (+z), or the first source's
+    // plane normal: an interface's (+z, its obliquity's own), or the first source's
     float e3x = 0.0f, e3y = 0.0f, e3z = 1.0f;
-    if (kind == RSI_STAGE_PISTON || normals == RSI_NORMALS_POINTS) {
+    if (kind == RSI_STAGE_PISTON) {
         const float nx = float(src.nx[first]), ny = float(src.ny[first]), nz = float(src.nz[first]);
         const float l2 = fmaf(nx, nx, fmaf(ny, ny, nz * nz));
         if (l2 > 0.25f && l2 < 4.0f) {
@@ -991,12 +991,11 @@ __device__ __forceinline__ void make_node(int kind, int normals, const PointsVie
     // extents (min, -max) along e1 and e2 turned by 0, 22.5, 45 and 67.5 degrees, and along e3
     const float ca[4] = {1.0f, 0.923879533f, 0.707106781f, 0.382683432f};
     const float sa[4] = {0.0f, 0.382683432f, 0.707106781f, 0.923879533f};
-    float ext[4][4], e3e[6] = {INFINITY, INFINITY, INFINITY, 0.f, 0.f, 0.f};  // min, -max along e3; -turn
+    float ext[4][4], e3e[6] = {INFINITY, INFINITY, 0.f, 0.f, 0.f, 0.f};  // min, -max along e3; -1: not a number
 #pragma unroll
     for (int r = 0; r < 4; ++r)
 #pragma unroll
         for (int d = 0; d < 4; ++d) ext[r][d] = INFINITY;
-    float turn = 0.0f;
     for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
         const int64_t j = rsi_fp32::source_slot(i, n, mode);
         float x, y, z, lo;
@@ -1012,12 +1011,8 @@ __device__ __forceinline__ void make_node(int kind, int normals, const PointsVie
             ext[r][2] = fminf(ext[r][2], b), ext[r][3] = fminf(ext[r][3], -b);
         }
         e3e[0] = fminf(e3e[0], s3), e3e[1] = fminf(e3e[1], -s3);
-        if (kind == RSI_STAGE_RSI && normals == RSI_NORMALS_POINTS)
-            turn = fmaxf(turn, fabsf(float(src.nx[j]) - e3x) + fabsf(float(src.ny[j]) - e3y) +
-                                   fabsf(float(src.nz[j]) - e3z));
-        if (!(isfinite(x) && isfinite(y) && isfinite(z))) turn = INFINITY;  // left to the direct sum
+        if (!(isfinite(x) && isfinite(y) && isfinite(z))) e3e[2] = -1.0f;  // left to the direct sum
     }
-    e3e[2] = -turn;
     float v[3][6];
 #pragma unroll
     for (int d = 0; d < 16; ++d) v[d / 6][d % 6] = ext[d / 4][d % 4];
@@ -1051,7 +1046,7 @@ __device__ __forceinline__ void make_node(int kind, int normals, const PointsVie
         df_diff(xh, xl, -c[0], 0.0f, o.c[0], o.c[1]);
         df_diff(yh, yl, -c[1], 0.0f, o.c[2], o.c[3]);
         df_diff(zh, zl, -c[2], 0.0f, o.c[4], o.c[5]);
-        o.flat = -e3e[2] <= 2e-7f ? 1.0f : 0.0f;
+        o.flat = e3e[2] == 0.0f ? 1.0f : 0.0f;
         *out = o;
     }
 }
