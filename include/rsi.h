@@ -152,7 +152,11 @@ enum rsi_stage_kind {
                                the first Rayleigh-Sommerfeld solution itself.  */
 };
 enum rsi_precision {
-    RSI_PREC_FP64 = 0, /* double precision throughout                          */
+    RSI_PREC_FP64 = 0, /* distance and phase in doubles; amplitudes, sine, cosine and
+                          products as pairs of floats (48 bits), a term off by
+                          some 2e-15 beside its phase's rounding; amplitudes below
+                          2^-100 of the largest of their tile (64 sources) count
+                          as 0.  Variant 1: every operation in doubles       */
     RSI_PREC_FP32C = 1 /* FP32 pair arithmetic; per (target, source tile) a
                           double-float reference distance and phase k R mod 2 pi;
                           compensated accumulation across tiles              */
@@ -176,7 +180,9 @@ typedef struct rsi_stage {
     int32_t tpt;       /* targets per thread (FP32C: 1, 2 or 4; FP64: 1); 0 = auto */
     int32_t splits;    /* source splits (>= 1); 0 = auto                          */
     int32_t variant;   /* FP32C distance update: 0 = auto, 1 = reciprocal, 2 = Newton,
-                          3 = Newton on two sources per packed f32x2 instruction */
+                          3 = Newton on two sources per packed f32x2 instruction;
+                          FP64: 1 = every operation in doubles, at a fifth of the
+                          speed, any other value = auto                        */
     int32_t reserved;
 } rsi_stage;
 

@@ -156,7 +156,7 @@ int make_plan(const rsi_stage& st, int64_t n_src, int64_t n_tgt, Plan& p, int ma
     } else {
         p.tpt = 1;
         if (st.tpt && st.tpt != 1) return rsi_fail(RSI_E_INVAL, "FP64 targets per thread must be 1");
-        p.variant = 0;
+        p.variant = st.variant == 1 ? 1 : 0;
     }
     p.n_tiles = int((n_src + p.S - 1) / p.S);
     p.tile_bytes = RSI_TILE_HDR_BYTES +

@@ -47,7 +47,8 @@ __global__ void __launch_bounds__(kThreads)
     const int64_t j = j_raw < a.n_tgt ? j_raw : a.n_tgt - 1;
     const double qx = a.tgt.x[j], qy = a.tgt.y[j], qz = a.tgt.z[j];
     for (int i = tid; i < kTabSize; i += kThreads) tab[i] = kTab.e[i];
-    const Wave w = make_wave(a.k);
+    Wave w = make_wave(a.k);
+    if (a.variant == 1) w.span = 0u;  // every term in doubles
 
     if (tid == 0) {
         for (int s = 0; s < RSI_PIPE_STAGES; ++s) mbar_init(smem_u32(&bars[s]), 1);
@@ -74,6 +75,7 @@ __global__ void __launch_bounds__(kThreads)
             break;
         }
         const double scale = *reinterpret_cast<const double*>(smem + buf * a.tile_bytes);
+        const double fast_scale = KIND == RSI_STAGE_PISTON ? scale : scale * w.k;
         const Record* rec = reinterpret_cast<const Record*>(smem + buf * a.tile_bytes + RSI_TILE_HDR_BYTES);
         for (int i0 = 0; i0 < a.S; i0 += 32) {
             DF sr = {0.0f, 0.0f}, si = {0.0f, 0.0f};
@@ -97,8 +99,8 @@ __global__ void __launch_bounds__(kThreads)
                     neu_add(im, scale * v.y);
                 }
             }
-            neu_add(re, scale * (double(sr.h) + double(sr.l)));
-            neu_add(im, scale * (double(si.h) + double(si.l)));
+            neu_add(re, fast_scale * (double(sr.h) + double(sr.l)));
+            neu_add(im, fast_scale * (double(si.h) + double(si.l)));
         }
         __syncthreads();
         if (tid == 0 && it + RSI_PIPE_STAGES < ntile) {
