@@ -178,11 +178,11 @@ int make_plan(const rsi_stage& st, int64_t n_src, int64_t n_tgt, Plan& p, int ma
         int64_t slots = int64_t(rsi_num_sms()) * occ;
         // minimise (waves x tiles per CTA), the time of the busiest SM, plus
         // the reduction: a CTA's tile takes S pairs per target at this GPU's
-        // pair rate (FP32C 1.4e12 / s over all slots), a split's partial sums 14
+        // pair rate (FP32C 1.4e12 / s over all slots, FP64 4.2e10), a split's partial sums 14
         // FP64 operations per target at 2 a cycle and SM, on as many SMs as the
         // reduction has CTAs.  2^16 x 2^14 (RSI, FP32C): 128 splits 744 + 137 us,
         // 14 splits 827 + 19 us; a 1000 x 3000 x 1073 chain 218 -> 150 us
-        const double tile_us = double(p.S) * threads * p.tpt * double(slots) / (fp32 ? 1.4e6 : 7.5e3);
+        const double tile_us = double(p.S) * threads * p.tpt * double(slots) / (fp32 ? 1.4e6 : 4.2e4);
         const double red_us = double(n_tgt) * 14.0 / (double(std::min<int64_t>(rsi_num_sms(), (n_tgt + 255) / 256)) * 4.1e3);
         double best_cost = INFINITY;
         splits = 1;
