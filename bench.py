@@ -17,6 +17,7 @@ bounded sample of the same workload on the host cores.
 from __future__ import annotations
 
 import argparse
+import ctypes
 import json
 import math
 import os
@@ -281,14 +282,43 @@ def multi_ops(kind: str, nf: int, harmonic: bool = False) -> dict:
             "fma_pipe": 10.0 / nf + 3.0 + 1.0}
 
 
-def clustered_roofline(roof: dict, kernel: str) -> dict:
-    """The line of a launch whose far clusters of sources and targets interact
-    through Chebyshev nodes (csrc/stage_cluster.cu): `achieved` counts the pairs
-    that it stands for, `peak` is the bound of a kernel that forms each of them, so
-    their ratio is what the clusters save and no share of the hardware."""
-    if roof["frac"] is None or roof["frac"] <= 1.05:
+def clusters_offered(rsi, st, n_src: int, n_tgt: int, ks=None) -> bool:
+    """Whether the library offers this stage (with ks: at several frequencies)
+    clusters: it then asks for more workspace than for the direct sum."""
+    def size(variant):
+        s = type(st).from_buffer_copy(st)
+        s.variant = variant
+        if ks is None:
+            return rsi.workspace_bytes(s, n_src, n_tgt)
+        kd = (ctypes.c_double * len(ks))(*ks)
+        return rsi.load().rsi_stage_multi_workspace_bytes(ctypes.byref(s), len(ks), kd, n_src, n_tgt)
+    return not st.variant and size(0) > size(3)
+
+
+def chain_offers_clusters(rsi, cfgs, multi: bool, variant: int = 0) -> bool:
+    """Whether one of the interface stages of these chains is offered clusters."""
+    for c in cfgs[:1] if multi else cfgs:
+        its = c["interfaces"]
+        n = [int(it["n"]) for it in its] + [int(c["grid"]["nx"]) * int(c["grid"]["nz"])]
+        for i, it in enumerate(its):
+            ks = [rsi.wavenumber(q["freq"], q["media"][i + 1]["c"]) for q in cfgs] if multi else None
+            st = rsi.stage_struct(rsi.STAGE_RSI, "fp32c", rsi.wavenumber(c["freq"], c["media"][i + 1]["c"]), 1.0,
+                                  rsi.NORMALS_Z if it["kind"] == "rect" else rsi.NORMALS_POINTS, variant=variant)
+            if clusters_offered(rsi, st, n[i], n[i + 1], ks):
+                return True
+    return False
+
+
+def clustered_roofline(roof: dict, kernel: str, offered: bool) -> dict:
+    """The line of launches that are offered clusters (csrc/stage_cluster.cu),
+    where far clusters of sources and targets interact through Chebyshev nodes:
+    `achieved` counts the pairs that they stand for, `peak` is the bound of a
+    kernel that forms each of them, so their ratio is what the clusters save and
+    no share of the hardware, on whichever side of 1 it lies."""
+    if not offered or roof["frac"] is None:
         return roof
-    return dict(roof, kernel=kernel, frac=None, direct_bound_ratio=roof["frac"],
+    return dict(roof, kernel=f"{kernel}, or {roof['kernel']} where the device's estimate favours it", frac=None,
+                direct_bound_ratio=roof["frac"],
                 note="achieved: pairs represented per second; peak: the bound of the direct kernel, which forms "
                      "every pair; the clustered kernel issues 0.5 of its slots (profiles/stage_cluster_kernels.md)")
 
@@ -610,7 +640,8 @@ def run_ours(args):
                 "rsi_kernel": {"achieved": achieved / 1e9, "avg_launch_ms": avg_s * 1e3, "launches": rsi_n},
                 "avg_launch_ms": pis_avg * 1e3, "launches": pis_n}
     if cfgs[0]["precision"] != "fp64":
-        roof = clustered_roofline(roof, "cluster_kernel<RSI> and leftover_kernel<RSI>")
+        roof = clustered_roofline(roof, "cluster_kernel<RSI> and leftover_kernel<RSI>",
+                                  chain_offers_clusters(rsi, cfgs, multi, args.variant))
     if cfgs[0]["precision"] != "fp64" and args.config == "c2" and roof["frac"] is not None:
         roof["traffic"] = recorded_traffic("stage_multi_kernel" if multi else "stage_fp32_kernel")
 
@@ -920,7 +951,9 @@ def run_two_medium_f1(args):
                  "achieved": achieved / 1e9, "peak": peak / 1e9, "unit": "Gpair/s",
                  "frac": achieved / peak, "traffic": None, "limiter": limiter, "launches": rsi_n,
                  "piston_kernel_gpair_s": pis_pairs / max(pis_ms * 1e-3, 1e-12) / 1e9},
-                "cluster_kernel<RSI> and leftover_kernel<RSI> (reflected + transmitted)"),
+                "cluster_kernel<RSI> and leftover_kernel<RSI> (reflected + transmitted)",
+                clusters_offered(rsi, rsi.stage_struct(rsi.STAGE_RSI, "fp32c", 1.0), int(cfg["interfaces"][0]["n"]),
+                                 nx * int(cfg["grid_water"]["nz"]))),
             "clocks": clk, "gpu_launches": launches, "gpu": torch.cuda.get_device_name(dev)}
     print(json.dumps(line), flush=True)
 
@@ -969,6 +1002,9 @@ def run_raytrace_f2(args):
     clk_hz = (clk["sm_mhz"] if clk and clk.get("sm_mhz") else 2070.0) * 1e6
     peak, limiter = alu_roofline("raytrace", n_sm, clk_hz)
     achieved = rt_pairs / (rt_ms * 1e-3)
+    size = [rsi.load().rsi_raytrace_workspace_bytes(ctypes.byref(rsi.raytrace_struct(cfg, newton=n)),
+                                                    int(cfg["piston"]["n"]), pixels) for n in (0, 1)]
+    offered = size[0] > size[1]  # a step count asks for the direct sum
     err = None
     path = os.path.join(os.path.dirname(os.path.abspath(__file__)), "tests", "golden", "f2_5MHz.json")
     if os.path.exists(path) and not args.small:
@@ -990,7 +1026,7 @@ def run_raytrace_f2(args):
                 {"bound": "alu", "kernel": "raytrace_kernel", "achieved": achieved / 1e9, "peak": peak / 1e9,
                  "unit": "Gpair/s", "frac": achieved / peak, "traffic": None, "limiter": limiter,
                  "ops_per_pair": OPS["raytrace"], "launches": rt_n},
-                "raytrace_cluster_kernel and raytrace_leftover_kernel"),
+                "raytrace_cluster_kernel and raytrace_leftover_kernel", offered),
             "clocks": clk, "gpu_launches": launches, "gpu": torch.cuda.get_device_name(dev)}
     print(json.dumps(line), flush=True)
 

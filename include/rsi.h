@@ -600,8 +600,10 @@ int rsi_nn_infer(const rsi_nn_net *net, const void *w16, const float *w32, const
 uint64_t rsi_launch_count(void);
 
 /* Per-kernel timing of the source x target kernels.  While enabled, every
- * rsi_propagate_stage and rsi_raytrace_field call brackets its main kernel
- * with CUDA events recorded on the call's stream.  rsi_timing_enable(1)
+ * rsi_propagate_stage, rsi_propagate_stage_multi and rsi_raytrace_field call
+ * brackets its main kernel -- the clustered and the direct one where the device
+ * chooses, after the tiles, the clusters and the estimate -- with CUDA events
+ * recorded on the call's stream.  rsi_timing_enable(1)
  * clears the record and starts; rsi_timing_enable(0) stops.
  * rsi_timing_read(kind, ...) synchronises with the recorded events and
  * returns, for the kernels of that kind (RSI_STAGE_PISTON, RSI_STAGE_RSI or

@@ -102,3 +102,11 @@ def test_fma_pipe_limit():
     o = bench.OPS["rsi"]
     assert o["fma_pipe"] / 128 < 0.8 * o["mufu"] / 16
     assert bench.alu_roofline("rsi", SM, CLK)[1] == "mufu"
+
+
+@pytest.mark.parametrize("frac", [0.87, 1.2, 7.4])
+def test_a_clustered_launch_is_no_share_of_the_hardware(frac):
+    roof = {"kernel": "direct", "frac": frac}
+    assert bench.clustered_roofline(roof, "clustered", False) == roof
+    got = bench.clustered_roofline(roof, "clustered", True)
+    assert got["frac"] is None and got["direct_bound_ratio"] == frac and "clustered" in got["kernel"]
