@@ -66,8 +66,7 @@ __device__ __forceinline__ void mma_bf16(float* c, const uint32_t* a, const uint
 
 // logistic sigmoid with the hardware's power of two and reciprocal (a few ulp; the
 // results are rounded to bf16), each flushing what lies below 2^-126 to 0, which
-// 1 + exp(-z) does not notice and the quotient reaches as its limit past z = -87:
-// 4 instructions, where __fdividef and __expf guard those ranges with 6 more.
+// 1 + exp(-z) does not notice and the quotient reaches as its limit past z = -87.
 __device__ __forceinline__ float sigmoidf_(float z) {
     float e, r;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(__fmul_rn(z, -1.4426950408889634f)));  // log2(e)

@@ -4,9 +4,9 @@
 // phase and 48-bit amplitudes (stage_fp64_body.cuh), summed in pairs of floats
 // over 32 terms and in doubles with Neumaier compensation over those.
 // 2^12 x 2^12 pairs of a piston stage: 2.08 ms with every operation in doubles
-// (54 double instructions per pair), 0.40 ms now with 9.7, 0.92 of what the
-// pipe's rate allows for them; of an interface stage 2.37 and 0.40 (per-point
-// normals, 3 operations more: 2.46 and 0.49).
+// (54 double instructions per pair), 0.40 ms now with 9.7, 0.91 of what the
+// pipe's rate allows for them; of an interface stage 2.36 and 0.41 (per-point
+// normals, 3 operations more: 2.45 and 0.50).
 #include <math.h>
 
 #include "stage_fp64_body.cuh"
