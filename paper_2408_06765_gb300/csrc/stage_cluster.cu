@@ -231,9 +231,10 @@ bool cluster_plan(int kind, int normals, int nf, int64_t n_src, int64_t n_tgt, i
     p.fill = float(std::min(1.0, double(blocks * p.splits * nf) / double(slots)));
     // With few blocks of targets a CTA's own time and the preparation decide, which
     // the estimate does not see.  Direct and clustered, ms: rays from 44069 points
-    // onto 8 blocks 2.07, 3.01; piston 65536 onto 9 0.50, 0.54, 30000 onto 24 0.60,
-    // 0.64; interface 120000 onto 9 0.90, 1.01, but 262144 onto 5, 64 roots for
-    // their CTAs, 1.04, 0.76 and 65536 onto 16 0.88, 0.75; rays from 16384 onto 32 2.32, 1.77
+    // onto 8 blocks 2.07, 3.01, from 30000 onto 16 2.31, 2.17, from 65536 onto 16 4.81,
+    // 2.84; piston 65536 onto 9 0.50, 0.54, 30000 onto 24 0.60, 0.64; interface 120000
+    // onto 9 0.90, 1.01, but 262144 onto 5, 64 roots for their CTAs, 1.04, 0.76, and
+    // 65536 onto 16 0.87, 0.14 to 0.78 by frequency and distance
     if (blocks < (kind == RSI_STAGE_PISTON ? 32 : 16) && roots < 64) return false;
     // The share of the direct sum's time (134.4 instructions per source and 256
     // targets, 9.2e11 per warp and second) that the estimate may reach: what is left
