@@ -200,9 +200,9 @@ size_t rsi_stage_workspace_bytes(const rsi_stage *st, int64_t n_src, int64_t n_t
  * the work says that this is faster; a pair of clusters is then interpolated to
  * 5e-8 of a term (root mean square; 5e-7 the largest over the random pairs that
  * the limits were fitted to), below the FP32 rounding of a pair, which a cluster's
- * sources then share: the error of a field is 1 to 1.3 times the direct sum's,
- * less than it where k times the tiles' size is large.  variant 3 asks for the
- * direct sum.
+ * sources then share: over 400 random sums the relative L2 error of a field was up
+ * to 7e-7 above the direct sum's (1e-7 to 3e-6), and below it where k times the
+ * tiles' size is large.  variant 3 asks for the direct sum.
  * src_sigma: complex [n_src] in the source set's slot order (RSI only; NULL
  * for PISTON).  tgt_field: complex [n_tgt] in the target set's slot order,
  * overwritten.  workspace: >= rsi_stage_workspace_bytes(...), 256-byte
